@@ -346,7 +346,7 @@ size_t hopm_backward_workspace_size(int order, const int64_t* dims, tvc_dtype dt
  * cut into items of about 2^20 elements (output ranges of the contraction,
  * row ranges of gx, slab/row rectangles of gA), largest tensors first, and
  * pulled by persistent blocks from an atomic counter.  (hopm_batched runs
- * one block per tensor.)
+ * one thread-block cluster per tensor.)
  * All pointers in a descriptor are device pointers, FP32, dense row-major.
  */
 typedef struct {
@@ -383,7 +383,7 @@ size_t tvc_batched_workspace_size(const tvc_batch_desc* descs, int count);
 
 /* Times the candidate block mappings (lanes per output) of the forward
  * contraction of rows v == 1 on the tensors of each such shape class of the
- * batch and keeps the fastest for later calls of tvc_batched / hopm_batched
+ * batch and keeps the fastest for later calls of tvc_batched
  * in this process; synchronises the stream.
  * workspace: tvc_batched_workspace_size(descs, count) bytes; a batch
  * uploaded on it before must be uploaded again (call without
@@ -392,7 +392,7 @@ tvc_status tvc_batched_autotune(const tvc_batch_desc* descs, int count, void* wo
                                 tvc_stream_t stream);
 
 /* `iters` Gauss-Seidel HOPM sweeps (Section 3, Algorithm 1's schedule) on
- * every tensor of the batch, one block per tensor; FP64 norms. */
+ * every tensor of the batch, one thread-block cluster per tensor; FP64 norms. */
 tvc_status hopm_batched(const hopm_batch_desc* descs, int count, int iters, int flags, void* workspace,
                         size_t ws_bytes, tvc_stream_t stream);
 size_t hopm_batched_workspace_size(const hopm_batch_desc* descs, int count);

@@ -653,7 +653,7 @@ class TVCBatch:
 
 
 class HOPMBatch:
-    """A batch of FP32 power methods (one block per tensor, `iters` sweeps)."""
+    """A batch of FP32 power methods (one thread-block cluster per tensor, `iters` sweeps)."""
 
     def __init__(self, items, iters):
         self.iters = int(iters)

@@ -1,16 +1,16 @@
-// Batched contractions, adjoints and power methods over many independent
-// FP32 tensors of uneven order and shape, each batch in one persistent
-// launch (the GPU counterpart of the paper's task-based execution, Section
-// 4.3, where many TVCs overlap instead of joining after each one).
+// Batched contractions and adjoints over many independent FP32 tensors of
+// uneven order and shape, each batch in one persistent launch (the GPU
+// counterpart of the paper's task-based execution, Section 4.3, where many
+// TVCs overlap instead of joining after each one); the batched power method
+// is in batched_hopm.cu.
 //
-// Contraction and adjoints: the host cuts every tensor (largest first) into
+// The host cuts every tensor (largest first) into
 // work items of about 2^20 elements (output ranges of the forward
 // contraction, slab x row rectangles of gx and gA) and uploads the
 // descriptors and items into the workspace; a persistent kernel of a few
 // blocks per SM pulls items from an atomic work counter.  gx items of one
 // tensor leave partial sums that the tensor's last item adds in a fixed
-// order.  Power methods: one block runs every sweep of one tensor.  With
-// TVC_BATCH_PREUPLOADED the descriptors of a previous call are reused and a
+// order.  With TVC_BATCH_PREUPLOADED the descriptors of a previous call are reused and a
 // call issues only a memset and one kernel, so it can be captured in a CUDA
 // graph and replayed.
 //
@@ -45,16 +45,6 @@ struct BItem {
   int gf;         // lanes per output of the forward contraction
   int gxk;        // gx items (slab ranges) of this tensor
   int64_t gxp;    // their partials: floats [gxp, gxp + gxk * nk) of the partial area (gxk > 1)
-};
-
-struct HItem {
-  const float* A;
-  int d;
-  int gsel[TVC_MAX_ORDER];
-  int64_t dims[TVC_MAX_ORDER];
-  float* x[TVC_MAX_ORDER];
-  double* lam;
-  int* status;
 };
 
 // ---------------------------------------------------- block-level routines
@@ -145,55 +135,6 @@ __device__ void blk_tvc(const float* __restrict__ A, int64_t u, int64_t nk, int6
   }
 }
 
-// The power method's two passes over A (v >= 2): where v is even and A is
-// 8-byte aligned each thread takes two adjacent outputs and loads pairs,
-// twice the bytes in flight per thread for the same sixteen rows (a block
-// of the register-held contraction streams at the rate its bytes in flight
-// allow); otherwise blk_tvc.
-__device__ void blk_tvc_pass(const float* __restrict__ A, int64_t u, int64_t nk, int64_t v,
-                             const float* __restrict__ x, float* __restrict__ y, int G) {
-  if (v % 2 != 0 || (reinterpret_cast<uintptr_t>(A) & 7) != 0) {
-    blk_tvc(A, u, nk, v, x, y, G);
-    return;
-  }
-  const int64_t uv2 = u * v / 2;  // output pairs
-  int64_t q2 = threadIdx.x;
-  if (q2 >= uv2) return;
-  const int64_t v2 = v / 2;
-  int64_t i = q2 / v2, l = 2 * (q2 - i * v2);
-  const int64_t di = kBBT / v2, dl = 2 * (kBBT - di * v2);
-  for (; q2 < uv2; q2 += kBBT) {
-    const float* p = A + i * nk * v + l;
-    float a0 = 0.0f, a1 = 0.0f;
-    int64_t jj = 0;
-    for (; jj + 16 <= nk; jj += 16, p += 16 * v) {
-      float2 av[16];
-#pragma unroll
-      for (int q = 0; q < 16; q++) av[q] = __ldcs(reinterpret_cast<const float2*>(p + q * v));
-#pragma unroll
-      for (int q = 0; q < 16; q++) {
-        const float xv = __ldg(x + jj + q);
-        a0 = __fmaf_rn(av[q].x, xv, a0);
-        a1 = __fmaf_rn(av[q].y, xv, a1);
-      }
-    }
-    for (; jj < nk; jj++, p += v) {
-      const float2 av = __ldcs(reinterpret_cast<const float2*>(p));
-      const float xv = __ldg(x + jj);
-      a0 = __fmaf_rn(av.x, xv, a0);
-      a1 = __fmaf_rn(av.y, xv, a1);
-    }
-    y[i * v + l] = a0;
-    y[i * v + l + 1] = a1;
-    i += di;
-    l += dl;
-    if (l >= v) {
-      l -= v;
-      i++;
-    }
-  }
-}
-
 // gA[(i*nk + j)*v + l] = gy[i*v + l] * x[j] over slabs i in [i0, i1) and
 // rows j in [j0, j1), with coalesced stores: threads own columns l (v >= 32)
 // or positions q = j*v + l of the slab (v < 32, whole slabs).
@@ -214,42 +155,6 @@ __device__ void blk_gA(const float* __restrict__ gy, const float* __restrict__ x
       for (int64_t i = i0; i < i1; i++) __stcs(gA + i * S + q, __ldg(gy + i * v + l) * xj);
     }
   }
-}
-
-// w[c] = prod_{m < nm} x_m[digit_m(c)]
-__device__ void blk_outer(float* w, int nm, const int64_t* dims, float* const* xs) {
-  int64_t len = 1;
-  for (int m = 0; m < nm; m++) len *= dims[m];
-  for (int64_t c = threadIdx.x; c < len; c += kBBT) {
-    int64_t rem = c;
-    float acc = 1.0f;
-    int64_t dig[TVC_MAX_ORDER];
-    for (int m = nm - 1; m >= 0; m--) {
-      dig[m] = rem % dims[m];
-      rem /= dims[m];
-    }
-    acc = xs[0][dig[0]];
-    for (int m = 1; m < nm; m++) acc *= xs[m][dig[m]];
-    w[c] = acc;
-  }
-}
-
-// x = z / ||z|| with the norm in FP64; returns the norm (all threads).
-__device__ double blk_normalize(const float* z, float* x, int64_t n, double* red) {
-  double s = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += kBBT) s = fma((double)z[i], (double)z[i], s);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int off = kBBT / 2; off > 0; off >>= 1) {
-    if ((int)threadIdx.x < off) red[threadIdx.x] += red[threadIdx.x + off];
-    __syncthreads();
-  }
-  const double sigma = sqrt(red[0]);
-  __syncthreads();
-  if (isfinite(sigma) && sigma > 0.0)
-    for (int64_t i = threadIdx.x; i < n; i += kBBT) x[i] = (float)((double)z[i] / sigma);
-  __syncthreads();
-  return sigma;
 }
 
 __device__ int grab(int* counter, int* slot) {
@@ -433,87 +338,6 @@ __global__ void __launch_bounds__(kBBT, 6) tvc_batched_kernel(const BItem* __res
   }
 }
 
-// One block runs every sweep of one tensor's power method (the schedule of
-// the single-tensor path: T = A x_1 x_1, W_1 = A x_0 x_0, W_j = W_{j-1} x_{j-1} ...,
-// the trailing contractions against the outer product of the trailing
-// vectors).  scratch: per block, 3 buffers of `slen` floats plus z.
-__global__ void __launch_bounds__(kBBT) hopm_batched_kernel(const HItem* __restrict__ items, int count, int iters,
-                                                            int* counter, float* scratch, int64_t slen, int64_t zlen) {
-  __shared__ int slot;
-  __shared__ double red[kBBT];
-  float* S1 = scratch + (int64_t)blockIdx.x * (3 * slen + zlen);
-  float* S2 = S1 + slen;
-  float* Wv = S2 + slen;
-  float* z = Wv + slen;
-  for (int b = grab(counter, &slot); b < count; b = grab(counter, &slot)) {
-    const HItem& it = items[b];
-    const int d = it.d;
-    const int64_t* n = it.dims;
-    int64_t N = 1;
-    for (int m = 0; m < d; m++) N *= n[m];
-    int status = TVC_OK;
-    double sigma = 0.0;
-    for (int t = 0; t < iters && status == TVC_OK; t++) {
-      float* prev = S1;
-      float* next = S2;
-      for (int j = 0; j < d && status == TVC_OK; j++) {
-        const float* zz = z;
-        if (d == 2) {
-          // z_j = A x_{1-j} x_{1-j}
-          if (j == 0)
-            blk_tvc(it.A, n[0], n[1], 1, it.x[1], z, it.gsel[1]);
-          else
-            blk_tvc(it.A, 1, n[0], n[1], it.x[0], z, it.gsel[0]);
-        } else if (j < 2) {
-          int64_t rest2 = 1;
-          for (int m = 2; m < d; m++) rest2 *= n[m];
-          if (j == 0)
-            blk_tvc_pass(it.A, n[0], n[1], rest2, it.x[1], S1, it.gsel[1]);  // T = A x_1 x_1
-          else
-            blk_tvc_pass(it.A, 1, n[0], N / n[0], it.x[0], S1, it.gsel[0]);  // W_1 = A x_0 x_0
-          __syncthreads();
-          const float* wvec = it.x[2];
-          if (d > 3) {
-            blk_outer(Wv, d - 2, n + 2, it.x + 2);
-            __syncthreads();
-            wvec = Wv;
-          }
-          blk_tvc(S1, n[j], rest2, 1, wvec, z, 32);
-          prev = S1;
-          next = S2;
-        } else {
-          int64_t rest = 1;
-          for (int m = j; m < d; m++) rest *= n[m];
-          blk_tvc(prev, 1, n[j - 1], rest, it.x[j - 1], next, 1);  // W_j = W_{j-1} x_{j-1}
-          __syncthreads();
-          if (j == d - 1) {
-            zz = next;
-          } else {
-            const float* wvec = it.x[d - 1];
-            if (j < d - 2) {
-              blk_outer(Wv, d - j - 1, n + j + 1, it.x + j + 1);
-              __syncthreads();
-              wvec = Wv;
-            }
-            blk_tvc(next, n[j], rest / n[j], 1, wvec, z, 32);
-          }
-          float* tmp = prev;
-          prev = next;
-          next = tmp;
-        }
-        __syncthreads();
-        sigma = blk_normalize(zz, it.x[j], n[j], red);
-        if (!isfinite(sigma)) status = TVC_ERR_NONFINITE;
-        else if (sigma == 0.0) status = TVC_ERR_ZERO_NORM;
-      }
-    }
-    if (threadIdx.x == 0) {
-      if (it.lam) *it.lam = sigma;
-      if (it.status) *it.status = status;
-    }
-  }
-}
-
 // ------------------------------------------------------------------ host --
 
 int64_t clog2(int64_t x) {
@@ -541,7 +365,6 @@ int pick_G(int64_t nk, int64_t v) {
 
 struct BLayout {
   size_t off_counter = 0, off_items = 0, off_scratch = 0, off_gxcnt = 0, off_gxpart = 0, total = 0;
-  int64_t slen = 0, zlen = 0;
   int blocks = 0;
 };
 
@@ -639,28 +462,6 @@ BLayout layout_tvc_items(const std::vector<BItem>& items, size_t nwork) {
   L.off_gxpart = L.off_gxcnt + align_up(items.size() * sizeof(int), 256);
   L.total = L.off_gxpart + align_up((size_t)std::max<int64_t>(1, nparts) * sizeof(float), 256);
   L.blocks = device_sms() * kBBlocksPerSM;
-  return L;
-}
-
-BLayout layout_hopm(const hopm_batch_desc* d, int count) {
-  BLayout L;
-  L.blocks = device_sms() * kBBlocksPerSM;
-  int64_t slen = 1, zlen = 1;
-  for (int b = 0; b < count; b++) {
-    int64_t N = 1, nmin = d[b].dims[0];
-    for (int m = 0; m < d[b].order; m++) {
-      N *= d[b].dims[m];
-      nmin = std::min(nmin, d[b].dims[m]);
-      zlen = std::max(zlen, d[b].dims[m]);
-    }
-    slen = std::max(slen, N / nmin);
-  }
-  L.slen = align_up((size_t)slen, 64);
-  L.zlen = align_up((size_t)zlen, 64);
-  L.off_counter = 0;
-  L.off_items = 256;
-  L.off_scratch = L.off_items + align_up((size_t)count * sizeof(HItem), 256);
-  L.total = L.off_scratch + (size_t)L.blocks * (3 * L.slen + L.zlen) * sizeof(float);
   return L;
 }
 
@@ -829,66 +630,5 @@ extern "C" tvc_status tvc_batched_autotune(const tvc_batch_desc* descs, int coun
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  return cuda_status(cudaGetLastError());
-}
-
-extern "C" size_t hopm_batched_workspace_size(const hopm_batch_desc* descs, int count) {
-  if (count < 0 || (count > 0 && !descs)) return 0;
-  for (int b = 0; b < count; b++)
-    if (descs[b].order < 2 || check_dims(descs[b].order, descs[b].dims, nullptr) != TVC_OK) return 0;
-  return layout_hopm(descs, count).total;
-}
-
-extern "C" tvc_status hopm_batched(const hopm_batch_desc* descs, int count, int iters, int flags, void* workspace,
-                                   size_t ws_bytes, tvc_stream_t stream) {
-  if (count < 0 || iters < 0 || !descs) return TVC_ERR_INVALID_ARG;
-  if (count == 0) return TVC_OK;
-  for (int b = 0; b < count; b++) {
-    if (descs[b].order < 2 || !descs[b].A || check_dims(descs[b].order, descs[b].dims, nullptr) != TVC_OK)
-      return TVC_ERR_INVALID_ARG;
-    for (int m = 0; m < descs[b].order; m++)
-      if (!descs[b].x[m]) return TVC_ERR_INVALID_ARG;
-  }
-  const BLayout L = layout_hopm(descs, count);
-  if (!workspace || ws_bytes < L.total) return TVC_ERR_WORKSPACE;
-  cudaStream_t st = (cudaStream_t)stream;
-  char* w = static_cast<char*>(workspace);
-  if (!(flags & TVC_BATCH_PREUPLOADED)) {
-    std::vector<std::pair<int64_t, int>> order;
-    for (int b = 0; b < count; b++) {
-      int64_t N = 1;
-      for (int m = 0; m < descs[b].order; m++) N *= descs[b].dims[m];
-      order.push_back({N, b});
-    }
-    std::stable_sort(order.begin(), order.end(), [](auto& a, auto& b) { return a.first > b.first; });
-    std::vector<HItem> items;
-    for (auto& pr : order) {
-      const hopm_batch_desc& e = descs[pr.second];
-      HItem it{};
-      it.A = e.A;
-      it.d = e.order;
-      for (int m = 0; m < e.order; m++) {
-        it.dims[m] = e.dims[m];
-        it.x[m] = e.x[m];
-      }
-      // lanes per output of the two big contractions (A x_1 x_1, A x_0 x_0)
-      int64_t N = 1;
-      for (int m = 0; m < e.order; m++) N *= e.dims[m];
-      it.gsel[0] = pick_G(e.dims[0], N / e.dims[0]);
-      it.gsel[1] = pick_G(e.dims[1], N / (e.dims[0] * e.dims[1]));
-      it.lam = e.lambda_out;
-      it.status = e.status_out;
-      items.push_back(it);
-    }
-    if (cudaMemcpyAsync(w + L.off_items, items.data(), items.size() * sizeof(HItem), cudaMemcpyHostToDevice, st) !=
-        cudaSuccess)
-      return TVC_ERR_CUDA;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return TVC_ERR_CUDA;
-  }
-  cudaMemsetAsync(w + L.off_counter, 0, sizeof(int), st);
-  hopm_batched_kernel<<<L.blocks, kBBT, 0, st>>>(reinterpret_cast<const HItem*>(w + L.off_items), count, iters,
-                                                reinterpret_cast<int*>(w + L.off_counter),
-                                                reinterpret_cast<float*>(w + L.off_scratch), L.slen, L.zlen);
-  count_launches(1);
   return cuda_status(cudaGetLastError());
 }
