@@ -4,13 +4,13 @@
 // TVCs overlap instead of joining after each one); the batched power method
 // is in batched_hopm.cu.
 //
-// The host cuts every tensor (largest first) into
-// work items of about 2^20 elements (output ranges of the forward
-// contraction, slab x row rectangles of gx and gA) and uploads the
+// The host cuts every tensor (largest first) into work items and uploads the
 // descriptors and items into the workspace; a persistent kernel of a few
-// blocks per SM pulls items from an atomic work counter.  gx items of one
-// tensor leave partial sums that the tensor's last item adds in a fixed
-// order.  With TVC_BATCH_PREUPLOADED the descriptors of a previous call are reused and a
+// blocks per SM pulls items from an atomic work counter.  Where a tensor
+// wants gx and another of its results, one item computes all of them for a
+// range of columns (v >= 32) or rows (v == 1) from one read of A; the other
+// cases have an item kind per result.  gx items of one tensor leave partial
+// sums that the tensor's last item adds in a fixed order.  With TVC_BATCH_PREUPLOADED the descriptors of a previous call are reused and a
 // call issues only a memset and one kernel, so it can be captured in a CUDA
 // graph and replayed.
 //
@@ -32,7 +32,7 @@ namespace tvcg {
 namespace {
 
 constexpr int kBBT = 256;        // threads per block
-constexpr int kBBlocksPerSM = 6;
+constexpr int kBBlocksPerSM = 4;
 
 struct BItem {
   const float* A;
@@ -48,6 +48,44 @@ struct BItem {
 };
 
 // ---------------------------------------------------- block-level routines
+
+// Rows [r0, r1) of a matrix of rows of nk elements against x: G lanes (a
+// power of two) per row, Q loads per lane and row and 16 / Q rows per group
+// in flight, shuffle reduction.
+template <int Q>
+__device__ void blk_rows(const float* __restrict__ A, int64_t nk, const float* __restrict__ x, float* __restrict__ y,
+                         int G, int64_t r0, int64_t r1) {
+  constexpr int B = 16 / Q;
+  const int lane = threadIdx.x & 31, p = lane & (G - 1), gw = 32 / G;
+  for (int64_t base = r0 + (int64_t)(threadIdx.x >> 5) * gw * B; base < r1; base += (int64_t)(kBBT / 32) * gw * B) {
+    const int64_t row0 = base + lane / G;
+    float acc[B];
+#pragma unroll
+    for (int b = 0; b < B; b++) acc[b] = 0.0f;
+    for (int64_t j = p; j - p < nk; j += Q * G) {
+      float av[B][Q], xv[Q];
+#pragma unroll
+      for (int q = 0; q < Q; q++) {
+        const bool in = j + q * G < nk;
+        xv[q] = in ? __ldg(x + j + q * G) : 0.0f;
+#pragma unroll
+        for (int b = 0; b < B; b++)
+          av[b][q] = (in && row0 + b * gw < r1) ? __ldcs(A + (row0 + b * gw) * nk + j + q * G) : 0.0f;
+      }
+#pragma unroll
+      for (int b = 0; b < B; b++)
+#pragma unroll
+        for (int q = 0; q < Q; q++) acc[b] = __fmaf_rn(av[b][q], xv[q], acc[b]);
+    }
+    for (int off = G / 2; off > 0; off >>= 1) {
+#pragma unroll
+      for (int b = 0; b < B; b++) acc[b] += __shfl_xor_sync(0xFFFFFFFFu, acc[b], off);
+    }
+#pragma unroll
+    for (int b = 0; b < B; b++)
+      if (p == 0 && row0 + b * gw < r1) y[row0 + b * gw] = acc[b];
+  }
+}
 
 // y[o] = sum_j A[(i*nk + j)*v + l] x[j], o = i*v + l < u*v; G lanes per output.
 __device__ void blk_tvc(const float* __restrict__ A, int64_t u, int64_t nk, int64_t v, const float* __restrict__ x,
@@ -107,32 +145,16 @@ __device__ void blk_tvc(const float* __restrict__ A, int64_t u, int64_t nk, int6
     }
     return;
   }
-  // v == 1 (rows): a group of G lanes per row, eight predicated loads in
-  // flight per lane (short rows too), shuffle reduction.
-  const int lane = threadIdx.x & 31;
-  const int p = lane & (G - 1);
-  const int gw = 32 / G;  // groups per warp
-  const int64_t ngroups = (int64_t)(kBBT / 32) * gw;
-  for (int64_t base = o_begin + (int64_t)(threadIdx.x >> 5) * gw; base < uv; base += ngroups) {
-    const int64_t o = base + lane / G;
-    float acc = 0.0f;
-    if (o < uv) {
-      const float* row = A + o * nk;
-      for (int64_t j = p; j < nk; j += 8 * G) {
-        float av[8], xv[8];
-#pragma unroll
-        for (int q = 0; q < 8; q++) {
-          const bool ok = j + q * G < nk;
-          av[q] = ok ? __ldcs(row + j + q * G) : 0.0f;
-          xv[q] = ok ? __ldg(x + j + q * G) : 0.0f;
-        }
-#pragma unroll
-        for (int q = 0; q < 8; q++) acc = __fmaf_rn(av[q], xv[q], acc);
-      }
-    }
-    for (int off = G / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
-    if (o < uv && p == 0) y[o] = acc;
-  }
+  // v == 1 (rows): a group of G lanes per row, Q loads per lane and row
+  const int64_t q = (nk + G - 1) / G;
+  if (q <= 1)
+    blk_rows<1>(A, nk, x, y, G, o_begin, uv);
+  else if (q <= 2)
+    blk_rows<2>(A, nk, x, y, G, o_begin, uv);
+  else if (q <= 4)
+    blk_rows<4>(A, nk, x, y, G, o_begin, uv);
+  else
+    blk_rows<8>(A, nk, x, y, G, o_begin, uv);
 }
 
 // gA[(i*nk + j)*v + l] = gy[i*v + l] * x[j] over slabs i in [i0, i1) and
@@ -148,11 +170,16 @@ __device__ void blk_gA(const float* __restrict__ gy, const float* __restrict__ x
         for (int64_t j = j0; j < j1; j++, p += v) __stcs(p, g * __ldg(x + j));
       }
   } else {
+    // columns q = j*v + l of the slab; slabs narrower than the block are
+    // written by several phases of threads
     const int64_t S = nk * v;
-    for (int64_t q = threadIdx.x; q < S; q += kBBT) {
+    const int CW = (int)min(S, (int64_t)kBBT), P = kBBT / CW;
+    const int ph = threadIdx.x / CW, cc = threadIdx.x - ph * CW;
+    for (int64_t q = cc; ph < P && q < S; q += CW) {
       const int64_t j = q / v, l = q - j * v;
       const float xj = __ldg(x + j);
-      for (int64_t i = i0; i < i1; i++) __stcs(gA + i * S + q, __ldg(gy + i * v + l) * xj);
+#pragma unroll 8
+      for (int64_t i = i0 + ph; i < i1; i += P) __stcs(gA + i * S + q, __ldg(gy + i * v + l) * xj);
     }
   }
 }
@@ -169,7 +196,9 @@ __device__ int grab(int* counter, int* slot) {
 // A unit of work: kind 0 = outputs [a0, a1) of the forward contraction,
 // 1 = gx over slabs [a0, a1) and rows j in [c0, c1) (slab range e0 of the
 // tensor's gxk, e1 gx items in all), 2 = gA over slabs [a0, a1) and rows
-// [c0, c1).
+// [c0, c1), 3 = every wanted result over the columns [a0, a1), 4 = every
+// wanted result over the rows i in [a0, a1) of v == 1 (e0, e1 as for gx), 5 =
+// gx and gA over a rectangle (v < 32).
 struct WItem {
   int b, kind;
   int64_t a0, a1, c0, c1;
@@ -195,8 +224,36 @@ struct WItem {
 // waiting.
 constexpr int64_t kGxWarpRows = 32;  // v at or above which rows go to warps
 constexpr int64_t kGxJ = 256;        // rows j per warp-mapped item
+constexpr int kFusedRows = 512;      // rows n_k up to which columns are fused
+constexpr int kFusedRowMax = 256;    // row lengths of the fused rows (v == 1)
+constexpr int kFusedRowMin = 32;
 
-__device__ void blk_gx_rect(const BItem& it, int64_t i0, int64_t i1, int64_t j0, int64_t j1, int ks, int items,
+
+// After an item's partial sums of gx are written: the tensor's last item
+// adds the gxk partials in order and resets the counter.
+__device__ void finish_gx(const BItem& it, int items, int* cnt, const float* partials, int* flag) {
+  if (it.gxk <= 1) return;
+  const int t = threadIdx.x;
+  __threadfence();
+  __syncthreads();
+  if (t == 0) *flag = (atomicAdd(cnt, 1) == items - 1);
+  __syncthreads();
+  if (*flag) {
+    __threadfence();
+    const float* Pp = partials + it.gxp;
+    for (int64_t j = t; j < it.nk; j += kBBT) {
+      KahanF32 sum;
+#pragma unroll 8
+      for (int q = 0; q < it.gxk; q++) sum.add(__ldcg(Pp + (int64_t)q * it.nk + j));
+      it.gx[j] = sum.value();
+    }
+    if (t == 0) *cnt = 0;  // ready for the next launch
+  }
+  __syncthreads();
+}
+
+// gA (nullable): rows of v < 32 also write gA over the rectangle.
+__device__ void blk_gx_rect(const BItem& it, float* __restrict__ gA, int64_t i0, int64_t i1, int64_t j0, int64_t j1, int ks, int items,
                             int* cnt, float* partials, float* red, int* flag) {
   const int64_t S = it.nk * it.v, v = it.v;
   float* dst = (it.gxk > 1) ? partials + it.gxp + (int64_t)ks * it.nk : it.gx;
@@ -262,9 +319,11 @@ __device__ void blk_gx_rect(const BItem& it, int64_t i0, int64_t i1, int64_t j0,
         const int64_t di = P;
         const float* a = it.A + (i0 + ph) * S + c;
         const float* g = it.gy + (i0 + ph) * v + l;
+        const float xj = gA ? __ldg(it.x + c / v) : 0.0f;
+        float* o = gA + (i0 + ph) * S + c;
         int64_t i = i0 + ph;
         int blk = 0;
-        for (; i + 7 * di < i1; i += 8 * di, a += 8 * di * S, g += 8 * di * v) {
+        for (; i + 7 * di < i1; i += 8 * di, a += 8 * di * S, g += 8 * di * v, o += 8 * di * S) {
           float av[8], gv[8];
 #pragma unroll
           for (int q = 0; q < 8; q++) {
@@ -272,14 +331,21 @@ __device__ void blk_gx_rect(const BItem& it, int64_t i0, int64_t i1, int64_t j0,
             gv[q] = __ldg(g + q * di * v);
           }
 #pragma unroll
-          for (int q = 0; q < 8; q++) acc = __fmaf_rn(av[q], gv[q], acc);
+          for (int q = 0; q < 8; q++) {
+            acc = __fmaf_rn(av[q], gv[q], acc);
+            if (gA) __stcs(o + q * di * S, gv[q] * xj);
+          }
           if (++blk == 8) {
             tot.add(acc);
             acc = 0.0f;
             blk = 0;
           }
         }
-        for (; i < i1; i += di, a += di * S, g += di * v) acc = __fmaf_rn(__ldcs(a), __ldg(g), acc);
+        for (; i < i1; i += di, a += di * S, g += di * v, o += di * S) {
+          const float gv = __ldg(g);
+          acc = __fmaf_rn(__ldcs(a), gv, acc);
+          if (gA) __stcs(o, gv * xj);
+        }
         tot.add(acc);
       }
       red[t] = (ph < P && cb + cc < C) ? tot.value() : 0.0f;
@@ -301,38 +367,270 @@ __device__ void blk_gx_rect(const BItem& it, int64_t i0, int64_t i1, int64_t j0,
       __syncthreads();
     }
   }
-  if (it.gxk > 1) {
-    __threadfence();
-    __syncthreads();
-    if (t == 0) *flag = (atomicAdd(cnt, 1) == items - 1);
-    __syncthreads();
-    if (*flag) {
-      __threadfence();
-      const float* Pp = partials + it.gxp;
-      for (int64_t j = t; j < it.nk; j += kBBT) {
-        KahanF32 sum;
-        for (int q = 0; q < it.gxk; q++) sum.add(__ldcg(Pp + (int64_t)q * it.nk + j));
-        it.gx[j] = sum.value();
-      }
-      if (t == 0) *cnt = 0;  // ready for the next launch
+  finish_gx(it, items, cnt, partials, flag);
+}
+
+// The sums over the warp's lanes of a[0..M-1], the kept values halved per
+// exchange (M = 16: 16 shuffles instead of 80): lane L returns the sum of
+// a[L / (32 / M)].
+template <int M>
+__device__ __forceinline__ float warp_add_many(float (&a)[M]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = M / 2, bit = 16; h >= 1; h >>= 1, bit >>= 1) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int e = 0; e < h; e++) {
+      const float mine = up ? a[e + h] : a[e], other = up ? a[e] : a[e + h];
+      a[e] = mine + __shfl_xor_sync(0xFFFFFFFFu, other, bit);
     }
-    __syncthreads();
+  }
+  float r = a[0];
+#pragma unroll
+  for (int bit = 16 / M; bit >= 1; bit >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, bit);
+  return r;
+}
+
+template <int VEC>
+__device__ __forceinline__ void ld_vec(const float* p, float (&v)[VEC]) {
+  if constexpr (VEC == 4) {
+    const float4 f = __ldcs(reinterpret_cast<const float4*>(p));
+    v[0] = f.x;
+    v[1] = f.y;
+    v[2] = f.z;
+    v[3] = f.w;
+  } else if constexpr (VEC == 2) {
+    const float2 f = __ldcs(reinterpret_cast<const float2*>(p));
+    v[0] = f.x;
+    v[1] = f.y;
+  } else {
+    v[0] = __ldcs(p);
   }
 }
 
-__global__ void __launch_bounds__(kBBT, 6) tvc_batched_kernel(const BItem* __restrict__ items,
+template <int VEC>
+__device__ __forceinline__ void st_vec(float* p, const float (&v)[VEC], float m) {
+  if constexpr (VEC == 4)
+    __stcs(reinterpret_cast<float4*>(p), make_float4(v[0] * m, v[1] * m, v[2] * m, v[3] * m));
+  else if constexpr (VEC == 2)
+    __stcs(reinterpret_cast<float2*>(p), make_float2(v[0] * m, v[1] * m));
+  else
+    __stcs(p, v[0] * m);
+}
+
+// y, gx and gA (those that are wanted) of the columns o = (i, l) in [c0, c1)
+// over all rows j, v >= 32: a thread owns four columns (VEC adjacent ones,
+// 4 / VEC pieces 32 VEC apart), holds their gy and y sums in registers and
+// walks the rows RB at a time: one load of A serves the column sum y += A x_j
+// and the row sum of A gy, which a warp reduces over its lanes per RB rows
+// into its own row of red; gA = gy x_j is written on the way.  Bound: one read
+// of A and one write of gA (three passes over memory with an item kind per
+// result).  512 tensors (2.1e9 elements) with all three results, with
+// blk_rows_fused and the smaller items: 7.89 -> 4.46 ms; 40 tensors 3.5 ->
+// 0.42 ms.
+template <int VEC>
+__device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, int items, int* cnt, float* partials,
+                               float* red, float* xsm, int* flag) {
+  constexpr int RB = VEC == 1 ? 16 : 8, NQ = 4 / VEC;
+  const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
+  const int nk = (int)it.nk;
+  const int64_t v = it.v;
+  const bool wy = it.y != nullptr, wgx = it.gx != nullptr, wgA = it.gA != nullptr;
+  const bool small = it.u * v <= 0xFFFFFFFFll;  // 32-bit division of the columns
+  float* const rw = red + wid * kFusedRows;
+  if (wy || wgA)
+    for (int j = t; j < nk; j += kBBT) xsm[j] = __ldg(it.x + j);
+  if (wgx)
+    for (int j = lane; j < nk; j += 32) rw[j] = 0.0f;
+  __syncthreads();
+  const int nbat = (nk + RB - 1) / RB, per = (nk + nbat - 1) / nbat;
+  for (int64_t g = c0 + wid * 128; g < c1; g += (kBBT / 32) * 128) {
+    int64_t off[NQ];
+    float gc[NQ][VEC], y0[NQ][VEC], y1[NQ][VEC];
+    const int64_t col0 = g + lane * VEC;
+#pragma unroll
+    for (int q = 0; q < NQ; q++) {
+      const int64_t col = col0 + q * 32 * VEC;
+      const bool ok = col < c1;
+      const int64_t i = small ? (int64_t)((uint32_t)col / (uint32_t)v) : col / v;
+      off[q] = (i * nk) * v + (col - i * v);
+#pragma unroll
+      for (int e = 0; e < VEC; e++) {
+        gc[q][e] = (ok && (wgx || wgA)) ? __ldg(it.gy + col + e) : 0.0f;
+        y0[q][e] = y1[q][e] = 0.0f;
+      }
+    }
+    for (int jb = 0; jb < nk; jb += per) {
+      const int nb = min(per, nk - jb);
+      float acc[RB];
+#pragma unroll
+      for (int e = 0; e < RB; e++) acc[e] = 0.0f;
+#pragma unroll
+      for (int q = 0; q < NQ; q++) {
+        const bool ok = col0 + q * 32 * VEC < c1;
+        if (wy || wgx) {
+          float a[RB][VEC];
+          const float* p = it.A + off[q];
+#pragma unroll
+          for (int e = 0; e < RB; e++, p += v) {
+#pragma unroll
+            for (int c = 0; c < VEC; c++) a[e][c] = 0.0f;
+            if (e < nb && ok) ld_vec<VEC>(p, a[e]);
+          }
+          if (wy) {
+#pragma unroll
+            for (int e = 0; e < RB; e += 2) {
+              const float xa = e < nb ? xsm[jb + e] : 0.0f, xb = e + 1 < nb ? xsm[jb + e + 1] : 0.0f;
+#pragma unroll
+              for (int c = 0; c < VEC; c++) {
+                if (e < nb) y0[q][c] = __fmaf_rn(a[e][c], xa, y0[q][c]);
+                if (e + 1 < nb) y1[q][c] = __fmaf_rn(a[e + 1][c], xb, y1[q][c]);
+              }
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < RB; e++)
+#pragma unroll
+            for (int c = 0; c < VEC; c++) acc[e] = __fmaf_rn(a[e][c], gc[q][c], acc[e]);
+        }
+        if (wgA && ok) {
+          float* p = it.gA + off[q];
+#pragma unroll
+          for (int e = 0; e < RB; e++, p += v)
+            if (e < nb) st_vec<VEC>(p, gc[q], xsm[jb + e]);
+        }
+        off[q] += per * v;
+      }
+      if (wgx) {
+        const float sum = warp_add_many<RB>(acc);
+        const int row = lane / (32 / RB);
+        if (lane % (32 / RB) == 0 && row < nb) rw[jb + row] += sum;
+        __syncwarp();
+      }
+    }
+    if (wy) {
+#pragma unroll
+      for (int q = 0; q < NQ; q++)
+        if (col0 + q * 32 * VEC < c1) {
+#pragma unroll
+          for (int e = 0; e < VEC; e++) it.y[col0 + q * 32 * VEC + e] = y0[q][e] + y1[q][e];
+        }
+    }
+  }
+  __syncthreads();
+  if (wgx) {
+    float* dst = (it.gxk > 1) ? partials + it.gxp + (int64_t)ks * nk : it.gx;
+    for (int j = t; j < nk; j += kBBT) {
+      KahanF32 sum;
+#pragma unroll
+      for (int w = 0; w < kBBT / 32; w++) sum.add(red[w * kFusedRows + j]);
+      dst[j] = sum.value();
+    }
+    finish_gx(it, items, cnt, partials, flag);
+  }
+  __syncthreads();
+}
+
+// The same for rows [i0, i1) of v == 1, 32 <= n_k <= 256: lanes own
+// the columns j of up to eight chunks (x_j and the column sums gx in
+// registers), a warp walks eight rows at a time and reduces their sums y.
+__device__ void blk_rows_fused(const BItem& it, int64_t i0, int64_t i1, int ks, int items, int* cnt, float* partials,
+                               float* red, int* flag) {
+  constexpr int RB = 8, NC = kFusedRowMax / 32;
+  const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
+  const int nk = (int)it.nk;
+  const bool wy = it.y != nullptr, wgx = it.gx != nullptr, wgA = it.gA != nullptr;
+  float xq[NC], cs[NC];
+#pragma unroll
+  for (int q = 0; q < NC; q++) {
+    xq[q] = ((wy || wgA) && q * 32 + lane < nk) ? __ldg(it.x + q * 32 + lane) : 0.0f;
+    cs[q] = 0.0f;
+  }
+  for (int64_t i = i0 + wid * RB; i < i1; i += (kBBT / 32) * RB) {
+    const int nb = (int)min((int64_t)RB, i1 - i);
+    float pe[RB], acc[RB];
+#pragma unroll
+    for (int e = 0; e < RB; e++) {
+      pe[e] = ((wgx || wgA) && e < nb) ? __ldg(it.gy + i + e) : 0.0f;
+      acc[e] = 0.0f;
+    }
+#pragma unroll
+    for (int q = 0; q < NC; q += 2) {
+      if (q * 32 < nk) {
+        float a[2][RB];
+        const float* p = it.A + i * nk + q * 32 + lane;
+        const bool ok0 = q * 32 + lane < nk, ok1 = q * 32 + 32 + lane < nk;
+        if (wy || wgx) {
+#pragma unroll
+          for (int e = 0; e < RB; e++) {
+            a[0][e] = (e < nb && ok0) ? __ldcs(p + e * nk) : 0.0f;
+            a[1][e] = (e < nb && ok1) ? __ldcs(p + e * nk + 32) : 0.0f;
+          }
+#pragma unroll
+          for (int h = 0; h < 2; h++)
+#pragma unroll
+            for (int e = 0; e < RB; e++) {
+              acc[e] = __fmaf_rn(a[h][e], xq[q + h], acc[e]);
+              cs[q + h] = __fmaf_rn(a[h][e], pe[e], cs[q + h]);
+            }
+        }
+        if (wgA) {
+          float* o = it.gA + i * nk + q * 32 + lane;
+#pragma unroll
+          for (int e = 0; e < RB; e++) {
+            if (e < nb && ok0) __stcs(o + e * nk, pe[e] * xq[q]);
+            if (e < nb && ok1) __stcs(o + e * nk + 32, pe[e] * xq[q + 1]);
+          }
+        }
+      }
+    }
+    if (wy) {
+      const float sum = warp_add_many<RB>(acc);
+      const int row = lane / (32 / RB);
+      if (lane % (32 / RB) == 0 && row < nb) it.y[i + row] = sum;
+    }
+  }
+  if (wgx) {
+#pragma unroll
+    for (int q = 0; q < NC; q++)
+      if (q * 32 + lane < nk) red[wid * kFusedRows + q * 32 + lane] = cs[q];
+    __syncthreads();
+    float* dst = (it.gxk > 1) ? partials + it.gxp + (int64_t)ks * nk : it.gx;
+    for (int j = t; j < nk; j += kBBT) {
+      KahanF32 sum;
+#pragma unroll
+      for (int w = 0; w < kBBT / 32; w++) sum.add(red[w * kFusedRows + j]);
+      dst[j] = sum.value();
+    }
+    finish_gx(it, items, cnt, partials, flag);
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kBBT, kBBlocksPerSM) tvc_batched_kernel(const BItem* __restrict__ items,
                                                            const WItem* __restrict__ work, int nwork, int* counter,
                                                            int* gx_counters, float* gx_partials) {
   __shared__ int slot;
-  __shared__ float red[(kBBT / 32) * kGxJ];
+  __shared__ float red[(kBBT / 32) * kFusedRows];
+  __shared__ __align__(16) float xsm[kFusedRows];
   __shared__ int last_flag;
   for (int w = grab(counter, &slot); w < nwork; w = grab(counter, &slot)) {
     const WItem wi = work[w];
     const BItem it = items[wi.b];
     if (wi.kind == 0)
       blk_tvc(it.A, it.u, it.nk, it.v, it.x, it.y, it.gf, wi.a0, wi.a1);
-    else if (wi.kind == 1)
-      blk_gx_rect(it, wi.a0, wi.a1, wi.c0, wi.c1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, &last_flag);
+    else if (wi.kind == 3) {
+      const uintptr_t al = reinterpret_cast<uintptr_t>(it.A) | reinterpret_cast<uintptr_t>(it.gA);
+      if (it.v % 4 == 0 && al % 16 == 0)
+        blk_cols_fused<4>(it, wi.a0, wi.a1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, xsm, &last_flag);
+      else if (it.v % 2 == 0 && al % 8 == 0)
+        blk_cols_fused<2>(it, wi.a0, wi.a1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, xsm, &last_flag);
+      else
+        blk_cols_fused<1>(it, wi.a0, wi.a1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, xsm, &last_flag);
+    } else if (wi.kind == 4)
+      blk_rows_fused(it, wi.a0, wi.a1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, &last_flag);
+    else if (wi.kind == 1 || wi.kind == 5)
+      blk_gx_rect(it, wi.kind == 5 ? it.gA : nullptr, wi.a0, wi.a1, wi.c0, wi.c1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, &last_flag);
     else
       blk_gA(it.gy, it.x, it.gA, it.nk, it.v, wi.a0, wi.a1, wi.c0, wi.c1);
   }
@@ -351,16 +649,12 @@ std::mutex g_tune_mu;
 std::map<std::pair<int, int>, int> g_tune;
 std::map<void*, int> g_nwork;  // work items uploaded per workspace
 
-int rule_G(int64_t nk, int64_t v) {  // lanes splitting n_k per forward output
-  if (v >= 32) return 1;
-  if (v >= 8) return 4;
-  return nk >= 64 ? 32 : 8;
-}
+int rule_G(int64_t nk) { return nk <= 64 ? 8 : nk <= 128 ? 16 : 32; }  // lanes per forward row (v == 1)
 
 int pick_G(int64_t nk, int64_t v) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tune.find({(int)clog2(v), (int)clog2(nk)});
-  return it != g_tune.end() ? it->second : rule_G(nk, v);
+  return it != g_tune.end() ? it->second : rule_G(nk);
 }
 
 struct BLayout {
@@ -368,58 +662,90 @@ struct BLayout {
   int blocks = 0;
 };
 
-// Work of about this many elements per item (a few MB): large tensors
-// spread over many blocks, small ones make a single item.
-constexpr int64_t kItemElems = 1 << 20;
-
 int64_t cdiv64(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-int64_t assign_gx(std::vector<BItem>* items);
+// Elements of A per work item: about eight items per resident block, so
+// that the last items of a small batch still fill the GPU (24..512 tensors
+// of 8..192 per mode with a fixed 2^20: 2.1-7.9 ms, most of it the last
+// items alone), within 2^15 .. 2^19 (an item still streams long runs).
+int64_t item_elems(const std::vector<BItem>& items) {
+  double total = 0.0;
+  for (const BItem& it : items) total += (double)it.u * it.nk * it.v;
+  const double per = total / ((double)device_sms() * kBBlocksPerSM * 8);
+  int64_t ie = 1 << 15;
+  while (ie < (1 << 19) && ie < per) ie *= 2;
+  return ie;
+}
 
-// Rectangle of a gx item: jr rows j by sr slabs, about kItemElems elements.
+// The fused item kind of a tensor (3: columns, 4: rows; 0: none): where one
+// read of A serves gx and another result, or gx alone in the column case.
+int fused_kind(const BItem& it) {
+  const int wanted = (it.y != nullptr) + (it.gx != nullptr) + (it.gA != nullptr);
+  if (it.v >= kGxWarpRows && it.nk <= kFusedRows && (it.gx || wanted > 1)) return 3;
+  if (it.v == 1 && it.nk >= kFusedRowMin && it.nk <= kFusedRowMax && wanted > 1) return 4;
+  return 0;
+}
+
+// Columns (kind 3) or rows (kind 4) per fused item.
+int64_t fused_per(const BItem& it, int64_t ie) {
+  if (it.v == 1) return std::min<int64_t>(1024, std::max<int64_t>(256, ie / it.nk / 256 * 256));
+  return std::max<int64_t>(1024, ie / it.nk / 1024 * 1024);
+}
+
+int64_t assign_gx(std::vector<BItem>* items, int64_t ie);
+
+// Rectangle of a gx item: jr rows j by sr slabs, about ie elements.
 // Warp-mapped rows (v >= 32) take every slab of a j before cutting the slabs
 // and keep 8 slabs (one per warp) where the tensor has them; column-mapped
 // rows take whole slab widths.
-void gx_rect(const BItem& it, int64_t* jr, int64_t* sr) {
+void gx_rect(const BItem& it, int64_t ie, int64_t* jr, int64_t* sr) {
   const int64_t v = std::max<int64_t>(1, it.v);
   if (v >= kGxWarpRows)  // whole slab ranges per j first; at most kGxJ rows, 8 slabs when there are
-    *jr = std::max<int64_t>(1, std::min<int64_t>(std::min(it.nk, kGxJ), kItemElems / std::max<int64_t>(1, it.u * v)));
+    *jr = std::max<int64_t>(1, std::min<int64_t>(std::min(it.nk, kGxJ), ie / std::max<int64_t>(1, it.u * v)));
   else  // whole slab widths first (coalesced columns)
-    *jr = std::max<int64_t>(1, std::min<int64_t>(it.nk, kItemElems / v));
-  *sr = std::max<int64_t>(1, std::min<int64_t>(it.u, kItemElems / (*jr * v)));
+    *jr = std::max<int64_t>(1, std::min<int64_t>(it.nk, ie / v));
+  *sr = std::max<int64_t>(1, std::min<int64_t>(it.u, ie / (*jr * v)));
   if (v >= kGxWarpRows) *sr = std::max(*sr, std::min<int64_t>(it.u, 8));
 }
 
-void make_work(std::vector<BItem>& items, std::vector<WItem>* work) {
-  assign_gx(&items);
+void make_work(std::vector<BItem>& items, int64_t ie, std::vector<WItem>* work) {
+  assign_gx(&items, ie);
   work->clear();
   for (int b = 0; b < (int)items.size(); b++) {
     const BItem& it = items[b];
     const int64_t uv = it.u * it.v;
+    if (const int kind = fused_kind(it)) {
+      const int64_t per = fused_per(it, ie);
+      int ks = 0;
+      for (int64_t o = 0; o < uv; o += per, ks++)
+        work->push_back({b, kind, o, std::min(uv, o + per), 0, 0, ks, (int)cdiv64(uv, per)});
+      continue;
+    }
+    const bool with_gA = it.gx && it.gA && it.v < kGxWarpRows;  // one pass for both
     if (it.y) {
-      const int64_t per = std::max<int64_t>(256, cdiv64(kItemElems, it.nk) / 256 * 256);
+      const int64_t per = std::max<int64_t>(256, cdiv64(ie, it.nk) / 256 * 256);
       for (int64_t o = 0; o < uv; o += per) work->push_back({b, 0, o, std::min(uv, o + per), 0, 0, 0, 0});
     }
     if (it.gx) {  // rectangles (see assign_gx), partials summed by the tensor's last item
       int64_t jr, sr;
-      gx_rect(it, &jr, &sr);
+      gx_rect(it, ie, &jr, &sr);
       const int nitems = (int)(cdiv64(it.u, sr) * cdiv64(it.nk, jr));
       int ks = 0;
       for (int64_t i = 0; i < it.u; i += sr, ks++)
         for (int64_t j = 0; j < it.nk; j += jr)
-          work->push_back({b, 1, i, std::min(it.u, i + sr), j, std::min(it.nk, j + jr), ks, nitems});
+          work->push_back({b, with_gA ? 5 : 1, i, std::min(it.u, i + sr), j, std::min(it.nk, j + jr), ks, nitems});
     }
-    if (it.gA) {
+    if (it.gA && !with_gA) {
       const int64_t S = it.nk * it.v;
       if (it.v >= 32) {
         // rectangles of slabs x rows
-        const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(it.nk, kItemElems / it.v));
-        const int64_t slabs = std::max<int64_t>(1, kItemElems / (rows * it.v));
+        const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(it.nk, ie / it.v));
+        const int64_t slabs = std::max<int64_t>(1, ie / (rows * it.v));
         for (int64_t i = 0; i < it.u; i += slabs)
           for (int64_t j = 0; j < it.nk; j += rows)
             work->push_back({b, 2, i, std::min(it.u, i + slabs), j, std::min(it.nk, j + rows), 0, 0});
       } else {
-        const int64_t slabs = std::max<int64_t>(1, kItemElems / S);
+        const int64_t slabs = std::max<int64_t>(1, ie / S);
         for (int64_t i = 0; i < it.u; i += slabs)
           work->push_back({b, 2, i, std::min(it.u, i + slabs), 0, it.nk, 0, 0});
       }
@@ -431,17 +757,21 @@ void make_work(std::vector<BItem>& items, std::vector<WItem>* work) {
 // count, from the same construction the call uses).
 tvc_status check_tvc_descs(const tvc_batch_desc* d, int count, std::vector<BItem>* items);
 
-// gx items per tensor (slab ranges of about kItemElems elements) and the
-// offsets of their partials; called on every item list before make_work.
-int64_t assign_gx(std::vector<BItem>* items) {
+// gx items per tensor (slab, column or row ranges of about ie elements) and
+// the offsets of their partials; called on every item list by make_work.
+int64_t assign_gx(std::vector<BItem>* items, int64_t ie) {
   int64_t off = 0;
   for (BItem& it : *items) {
     it.gxk = 0;
     it.gxp = 0;
     if (!it.gx) continue;
-    int64_t jr, sr;
-    gx_rect(it, &jr, &sr);
-    it.gxk = (int)cdiv64(it.u, sr);
+    if (fused_kind(it)) {
+      it.gxk = (int)cdiv64(it.u * it.v, fused_per(it, ie));
+    } else {
+      int64_t jr, sr;
+      gx_rect(it, ie, &jr, &sr);
+      it.gxk = (int)cdiv64(it.u, sr);
+    }
     if (it.gxk > 1) {
       it.gxp = off;
       off += (int64_t)it.gxk * it.nk;
@@ -512,7 +842,7 @@ extern "C" size_t tvc_batched_workspace_size(const tvc_batch_desc* descs, int co
   std::vector<BItem> items;
   if (check_tvc_descs(descs, count, &items) != TVC_OK) return 0;
   std::vector<WItem> work;
-  make_work(items, &work);
+  make_work(items, item_elems(items), &work);
   return layout_tvc_items(items, work.size()).total;
 }
 
@@ -524,7 +854,7 @@ extern "C" tvc_status tvc_batched(const tvc_batch_desc* descs, int count, int fl
   tvc_status rc = check_tvc_descs(descs, count, &items);
   if (rc != TVC_OK) return rc;
   std::vector<WItem> work;
-  make_work(items, &work);
+  make_work(items, item_elems(items), &work);
   const BLayout L = layout_tvc_items(items, work.size());
   if (!workspace || ws_bytes < L.total) return TVC_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
@@ -570,7 +900,8 @@ extern "C" tvc_status tvc_batched_autotune(const tvc_batch_desc* descs, int coun
   tvc_status rc = check_tvc_descs(descs, count, &items);
   if (rc != TVC_OK) return rc;
   std::vector<WItem> allwork;
-  make_work(items, &allwork);
+  const int64_t ie = item_elems(items);
+  make_work(items, ie, &allwork);
   const BLayout L = layout_tvc_items(items, allwork.size());
   if (!workspace || ws_bytes < L.total) return TVC_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
@@ -593,11 +924,12 @@ extern "C" tvc_status tvc_batched_autotune(const tvc_batch_desc* descs, int coun
     std::vector<BItem> sub = kv.second;  // at most 256 tensors of the class
     if (sub.size() > 256) sub.resize(256);
     float best = 1e30f;
-    int bestG = rule_G(sub[0].nk, sub[0].v);
+    int bestG = rule_G(sub[0].nk);
     for (int G : cands) {
       for (BItem& it : sub) it.gf = G;
       std::vector<WItem> wk;
-      make_work(sub, &wk);
+      make_work(sub, ie, &wk);
+      if (wk.size() > allwork.size()) break;  // the workspace holds allwork
       cudaMemcpy(w + L.off_items, sub.data(), sub.size() * sizeof(BItem), cudaMemcpyHostToDevice);
       cudaMemcpy(w + L.off_scratch, wk.data(), wk.size() * sizeof(WItem), cudaMemcpyHostToDevice);
       float tot = 0.0f;
