@@ -39,29 +39,6 @@ constexpr int kThreads = 256;
 constexpr int kWarpsPerBlock = kThreads / kWarp;
 constexpr int kRB = 64;  // additions per accumulator between folds
 
-// x entries j .. j+VEC-1 (j a multiple of VEC): 16-byte loads when x is
-// 16-byte aligned and no per-row slab scale applies (k > 0), else one by one.
-template <tvc_dtype DT, int VEC>
-__device__ __forceinline__ void xvec(const TvcArgs<DT>& a, int64_t j, float (&xq)[VEC]) {
-  const float* x = static_cast<const float*>(a.x);
-  const bool fold = kNarrow<DT> && a.mode0 && a.scales;
-  if constexpr (VEC % 4 == 0) {
-    if (!fold && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
-#pragma unroll
-      for (int e = 0; e < VEC; e += 4) {
-        const float4 f = __ldg(reinterpret_cast<const float4*>(x + j + e));
-        xq[e] = f.x;
-        xq[e + 1] = f.y;
-        xq[e + 2] = f.z;
-        xq[e + 3] = f.w;
-      }
-      return;
-    }
-  }
-#pragma unroll
-  for (int e = 0; e < VEC; e++) xq[e] = xval(a, j + e);
-}
-
 // ------------------------------------------------------------------ COLS --
 
 template <tvc_dtype DT, int VEC, int DROWS>
@@ -1385,7 +1362,9 @@ enum Kind {
   K_TILE_ASYNC = 8,
   K_SLAB_ASYNC = 9,
   K_F64_TILE = 10,
-  K_SLAB_TILE = 11
+  K_SLAB_TILE = 11,
+  K_COLS_RAGGED = 12,
+  K_ROWS_RAGGED = 13
 };
 
 struct Plan {
@@ -1393,7 +1372,7 @@ struct Plan {
   int vec = 1;
   int64_t splits = 1, chunk = 0;
   int R = 0, vec16 = 0, g = 0, G = 0, nst = 0, RW = 0, S = 0, dq = 0, rb = 0, unr = 0;
-  int64_t ntiles = 0;
+  int64_t ntiles = 0, pps = 0;
   uint32_t tile_bytes = 0;
   size_t smem = 0;
   dim3 grid;
@@ -1611,6 +1590,43 @@ static bool plan_slab_tile(Plan& p, const Shape& s, tvc_dtype dt, int sms) {
   return true;
 }
 
+// Rows (v == 1) off 16-byte boundaries that go to the ragged row kernel: of
+// at least 16 bytes (shorter ones measured no faster there), but for FP32
+// rows of 13 to 15 elements (staged 3920 GB/s, here 3706).
+static bool rows_ragged_wanted(int64_t nk, size_t es) {
+  const int64_t bytes = nk * (int64_t)es;
+  return bytes >= 16 && !(es == 4 && bytes > 48 && bytes < 64);
+}
+
+static void plan_rows_ragged(Plan& p, const Shape& s, size_t es, int sms) {
+  p.kind = K_ROWS_RAGGED;
+  const int64_t vec = 16 / (int64_t)es, ppr = ceil_div(s.nk, vec);
+  // Lanes per row: the widest group whose lanes have at least four pieces
+  // each and 85% of them a piece in the last step, else the narrower group
+  // that leaves the fewest without; one lane only for rows of up to four
+  // pieces (rows of 76 bytes: 2494 GB/s alone, 4193 in pairs; of 33 E4M3
+  // elements 2328 alone).  Fewer pieces per lane leave the reduction of the
+  // lanes uncovered: E4M3 rows of 501 969 GB/s with 32 lanes, 2592 with 8.
+  int64_t best = INT64_MAX;
+  p.G = ppr <= 4 ? 1 : 2;
+  for (int G = 32; G >= 2 && ppr > 4; G /= 2) {
+    if (ppr < 4 * G && G > 2) continue;
+    const int64_t padded = ceil_div(ppr, G) * G;
+    if (padded < best) {
+      best = padded;
+      p.G = G;
+    }
+    if (100 * ppr >= 85 * padded) break;
+  }
+  const int64_t gw = kWarp / p.G, step = p.G * vec;
+  const int64_t warps = ceil_div(s.u, gw * kRaggedRowBatch), target = (int64_t)sms * 32;
+  int64_t splits = 1;
+  if (warps < target) splits = std::min(ceil_div(target, warps), std::max<int64_t>(1, s.nk / (4 * step)));
+  p.chunk = ceil_div(ceil_div(s.nk, splits), step) * step;
+  p.splits = ceil_div(s.nk, p.chunk);
+  p.grid = dim3((unsigned)ceil_div(warps, kWarpsPerBlock), (unsigned)p.splits);
+}
+
 static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool allow_staged) {
   Plan p;
   const bool f64acc = (dt == TVC_F64 || dt == TVC_F32D);  // FP64 arithmetic (float-float kernels)
@@ -1618,10 +1634,12 @@ static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool all
   const int64_t target_threads = (int64_t)sms * 2048;
   const int64_t S = s.nk * s.v;
   const size_t es = elem_size(dt);
+  const bool ragged = dt != TVC_F64 && dt != TVC_F32D && pick_vec(dt, s.v == 1 ? s.nk : s.v, A) * (int)es < 16;
   if (s.v >= 32) {
-    p.kind = K_COLS;
+    p.kind = ragged ? K_COLS_RAGGED : K_COLS;
     p.vec = pick_vec(dt, s.v, A);
-    const int64_t threads = ceil_div(s.uv, p.vec);
+    p.pps = ceil_div(s.v * (int64_t)es, 16);
+    const int64_t threads = ragged ? s.u * p.pps : ceil_div(s.uv, p.vec);
     int64_t splits = 1;
     if (threads < target_threads) splits = std::min(ceil_div(target_threads, threads), std::max<int64_t>(1, s.nk / 64));
     p.chunk = ceil_div(ceil_div(s.nk, splits), 8) * 8;
@@ -1629,6 +1647,8 @@ static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool all
     p.grid = dim3((unsigned)ceil_div(threads, kThreads), (unsigned)p.splits);
   } else if (dt == TVC_F64 && aligned(A, 16) && s.v < 32 && plan_f64_tile(p, s, sms)) {
     // FP64 small slabs and short rows: the copy-engine tile kernel.
+  } else if (s.v == 1 && !f64acc && ragged && rows_ragged_wanted(s.nk, es)) {
+    plan_rows_ragged(p, s, es, sms);
   } else if (s.v == 1 && !f64acc && allow_staged && aligned(A, 16) &&
              s.nk <= 8 * 32 * (int64_t)pick_vec(dt, s.nk, A, 4) && s.u >= 8) {
     // Staged short rows: tiles of R = 8*RW whole rows through shared memory.
@@ -1931,6 +1951,12 @@ static bool launch_main(const Plan& p, const TvcArgs<DT>& a, cudaStream_t st) {
       }
       break;
     }
+    case K_COLS_RAGGED:
+      if constexpr (!kF64Acc<DT>) cols_ragged_launch<DT>(a, p.grid, p.pps, st);
+      break;
+    case K_ROWS_RAGGED:
+      if constexpr (!kF64Acc<DT>) rows_ragged_launch<DT>(a, p.grid, p.G, st);
+      break;
     case K_ROWS:
       launch_rows<DT>(p, a, st);
       break;

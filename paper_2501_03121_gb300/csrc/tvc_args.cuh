@@ -67,6 +67,29 @@ __device__ __forceinline__ float xval(const TvcArgs<DT>& a, int64_t j) {
   return xv;
 }
 
+// x entries j .. j+VEC-1 (j a multiple of VEC): 16-byte loads when x is
+// 16-byte aligned and no per-row slab scale applies (k > 0), else one by one.
+template <tvc_dtype DT, int VEC>
+__device__ __forceinline__ void xvec(const TvcArgs<DT>& a, int64_t j, float (&xq)[VEC]) {
+  const float* x = static_cast<const float*>(a.x);
+  const bool fold = kNarrow<DT> && a.mode0 && a.scales;
+  if constexpr (VEC % 4 == 0) {
+    if (!fold && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
+#pragma unroll
+      for (int e = 0; e < VEC; e += 4) {
+        const float4 f = __ldg(reinterpret_cast<const float4*>(x + j + e));
+        xq[e] = f.x;
+        xq[e + 1] = f.y;
+        xq[e + 2] = f.z;
+        xq[e + 3] = f.w;
+      }
+      return;
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < VEC; e++) xq[e] = xval(a, j + e);
+}
+
 // Scale of output row i (k > 0): all elements of an output share slab i / upi0.
 template <tvc_dtype DT>
 __device__ __forceinline__ float out_scale(const TvcArgs<DT>& a, int64_t i) {
@@ -132,5 +155,15 @@ void slabtile_launch(const TvcArgs<TVC_BF16>& a, const SlabTileParams& prm, dim3
 void slabtile_launch(const TvcArgs<TVC_F16>& a, const SlabTileParams& prm, dim3 grid, cudaStream_t st);
 void slabtile_launch(const TvcArgs<TVC_E4M3>& a, const SlabTileParams& prm, dim3 grid, cudaStream_t st);
 tvc_status slabtile_device_error(int* code_out, int clear);
+
+// Rows that do not start on 16-byte boundaries (tvc_ragged.cu): columns
+// (v >= 32; FP32 accumulation; pps = ceil(v * element size / 16) pieces
+// per row) and rows (v == 1; FP32 accumulation; G lanes per row,
+// kRaggedRowBatch rows per group, chunk a multiple of G 16-byte pieces).
+constexpr int kRaggedRowBatch = 4;
+template <tvc_dtype DT>
+void cols_ragged_launch(const TvcArgs<DT>& a, dim3 grid, int64_t pps, cudaStream_t st);
+template <tvc_dtype DT>
+void rows_ragged_launch(const TvcArgs<DT>& a, dim3 grid, int G, cudaStream_t st);
 
 }  // namespace tvcg
