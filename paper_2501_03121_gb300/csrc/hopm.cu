@@ -349,7 +349,7 @@ struct Ctx {
 
 // Workspace layout of a forward run.
 struct FwdLayout {
-  size_t off_state = 0, off_bufA = 0, off_bufB = 0, off_w = 0, off_z = 0, off_tvc = 0, total = 0, tvc = 0;
+  size_t off_state = 0, off_bufA = 0, off_bufB = 0, off_w = 0, off_z = 0, off_tvc = 0, off_grid = 0, total = 0, tvc = 0;
 };
 
 FwdLayout fwd_layout(int order, const int64_t* dims, tvc_dtype dt, size_t base) {
@@ -384,6 +384,8 @@ FwdLayout fwd_layout(int order, const int64_t* dims, tvc_dtype dt, size_t base) 
   L.off_tvc = off;
   L.tvc = c.tvc_need;
   off += align_up(c.tvc_need, 256);
+  L.off_grid = off;
+  if (hopm_grid_wanted(order, dims, dt)) off += hopm_grid_ws_bytes(order, dims, dt);
   L.total = off;
   return L;
 }
@@ -423,6 +425,11 @@ tvc_status hopm_launch(const void* A, int order, const int64_t* dims, void* cons
   if (ws == nullptr || ws_bytes < L.total) return TVC_ERR_WORKSPACE;
   Ctx c;
   bind(c, L, ws, A, order, dims, dt, scales, st);
+  if (hopm_grid_wanted(order, dims, dt)) {
+    const tvc_status rc = hopm_grid_launch(A, order, dims, x, iters, tol, lam_out, sweeps_out, status_out, lam_hist, dt,
+                                           scales, c.bufA, c.bufB, static_cast<char*>(ws) + L.off_grid, st);
+    if (rc != TVC_ERR_UNSUPPORTED) return rc;
+  }
   c.init_state();
   for (int it = 0; it < iters && c.rc == TVC_OK; it++) c.sweep(x, tol, lam_out, sweeps_out, status_out, lam_hist, nullptr);
   count_launches(c.launches);
@@ -477,6 +484,9 @@ tvc_status dhopm_launch(const void* const* slabs, int parts, const int64_t* star
                         size_t ws_bytes, cudaStream_t st) {
   const DLayout D = dhopm_layout(parts, starts, order, dims, s, dt);
   if (ws == nullptr || ws_bytes < D.total) return TVC_ERR_WORKSPACE;
+  if (parts == 1)  // the unsplit method
+    return hopm_launch(slabs[0], order, dims, x, iters, tol, lam_out, sweeps_out, status_out, lam_hist, dt, scales, ws,
+                       ws_bytes, st);
   char* w = static_cast<char*>(ws);
   const size_t vs = vec_size(dt);
   Ctx g;  // global view: the state, the normalisation of the combined z

@@ -63,6 +63,18 @@ tvc_status tvc_launch(const void* A, const Shape& s, const void* x, void* y, tvc
                       cudaStream_t stream, const int* done = nullptr);
 size_t tvc_ws_bytes(const Shape& s, tvc_dtype dt, const void* A);
 
+// A whole power method in one cooperative launch (hopm_grid.cu), for tensors
+// where launches set the time: wanted says whether the sizes fit and pay,
+// ws_bytes what it needs beside the T and W_j buffers.  TVC_ERR_UNSUPPORTED:
+// nothing launched, the device cannot hold the grid at once.
+bool hopm_grid_wanted(int order, const int64_t* dims, tvc_dtype dt);
+size_t hopm_grid_ws_bytes(int order, const int64_t* dims, tvc_dtype dt);
+tvc_status hopm_grid_launch(const void* A, int order, const int64_t* dims, void* const* x, int iters, double tol,
+                            double* lam_out, int* sweeps_out, int* status_out, double* lam_hist, tvc_dtype dt,
+                            const float* scales, void* bufA, void* bufB, void* ws, cudaStream_t st);
+// Sticky error word of its grid barrier (cleared when clear != 0).
+tvc_status hopm_grid_device_error(int* code_out, int clear);
+
 // 1D split over virtual ranks (split.cu).  check_split validates parts,
 // starts and s against the tensor; slab_dims gives rank r's dims.
 tvc_status check_split(int parts, const int64_t* starts, int order, const int64_t* dims, int s);

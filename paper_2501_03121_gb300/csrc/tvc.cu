@@ -2102,6 +2102,8 @@ extern "C" tvc_status tvc_device_error(int* code_out, int clear) {
   if (v == 0 && w != 0) v = 20 + w;  // the FP64 tile kernel's waits
   if (slabtile_device_error(&w, clear) != TVC_OK) return TVC_ERR_CUDA;
   if (v == 0 && w != 0) v = 30 + w;  // the slab tile kernel's waits
+  if (hopm_grid_device_error(&w, clear) != TVC_OK) return TVC_ERR_CUDA;
+  if (v == 0 && w != 0) v = w;  // the power method's grid barrier
   if (code_out) *code_out = v;
   return v ? TVC_ERR_TIMEOUT : TVC_OK;
 }
