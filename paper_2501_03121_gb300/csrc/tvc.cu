@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <mutex>
 #include <set>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -1348,6 +1349,48 @@ __global__ void tvc_reduce_kernel(const V* __restrict__ partial, V* __restrict__
   }
 }
 
+// The same for few outputs and many splits: a block adds 32 outputs, each of
+// its 32 warps a contiguous share of the splits in order, then the warps'
+// sums in warp order (9710 splits of 128 outputs: 640 us with a thread per
+// output).
+template <class V>
+__global__ void __launch_bounds__(1024) tvc_reduce_many_kernel(const V* __restrict__ partial, V* __restrict__ y,
+                                                               int64_t uv, int64_t splits, double alpha, double beta,
+                                                               const int* done) {
+  if (skip(done)) return;
+  __shared__ V sums[32][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t o = (int64_t)blockIdx.x * 32 + lane;
+  const int64_t k0 = splits * w / 32, k1 = splits * (w + 1) / 32;
+  using Sum = std::conditional_t<sizeof(V) == 8, double, KahanF32>;
+  Sum s{};
+  auto add = [](Sum& t, V v) {
+    if constexpr (sizeof(V) == 8)
+      t += v;
+    else
+      t.add(v);
+  };
+  auto value = [](const Sum& t) -> V {
+    if constexpr (sizeof(V) == 8)
+      return t;
+    else
+      return t.value();
+  };
+  if (o < uv) {
+#pragma unroll 8
+    for (int64_t k = k0; k < k1; k++) add(s, partial[k * uv + o]);
+  }
+  sums[w][lane] = value(s);
+  __syncthreads();
+  if (w == 0 && o < uv) {
+    Sum t{};
+    for (int k = 0; k < 32; k++) add(t, sums[k][lane]);
+    V r = (V)alpha * value(t);
+    if (beta != 0.0) r += (V)beta * y[o];
+    y[o] = r;
+  }
+}
+
 // ------------------------------------------------------------------ plan --
 
 enum Kind {
@@ -1364,7 +1407,8 @@ enum Kind {
   K_F64_TILE = 10,
   K_SLAB_TILE = 11,
   K_COLS_RAGGED = 12,
-  K_ROWS_RAGGED = 13
+  K_ROWS_RAGGED = 13,
+  K_COLS_PHASED = 14
 };
 
 struct Plan {
@@ -1379,7 +1423,7 @@ struct Plan {
   F64TileParams ft{};
   SlabTileParams st{};
   int xs_shift = 0;  // FP64 rows of odd length with 16-byte pairs: the shifted split x too
-  size_t ws_xs = 0, ws_partial = 0, ws_total = 0;
+  size_t ws_xs = 0, ws_partial = 0, ws_least = 0, ws_total = 0;  // ws_least: of ws_partial
 };
 
 // Opts a kernel in to `bytes` of dynamic shared memory, once per kernel and
@@ -1627,6 +1671,62 @@ static void plan_rows_ragged(Plan& p, const Shape& s, size_t es, int sms) {
   p.grid = dim3((unsigned)ceil_div(warps, kWarpsPerBlock), (unsigned)p.splits);
 }
 
+// Columns that go to the phased kernel: few outputs over many rows, and
+// tensors of at most 12 MB, where latency sets the time (128^3 mode 0: FP32
+// 9.0 -> 5.1 us, BF16 10.5 -> 4.6, E4M3 13.4 -> 4.0; 300x70x33 FP64 12.9 ->
+// 7.3).  Between the two the column kernels stream longer runs per thread and
+// stay faster (FP32 1000x1000x100 mode 0 68 us, phased 110; 16 MB FP64 10.5,
+// phased 12.7).
+// The workspace stays at least what the column kernels would take, so that
+// callers who lend a fixed scratch keep the limits they had.
+constexpr int64_t kPhasedSmall = 12 << 20;
+
+static void set_phased(Plan& p, const Shape& s, tvc_dtype dt, const void* A, int w, int64_t splits) {
+  const int64_t es = (int64_t)elem_size(dt);
+  p.ws_least = p.splits > 1 ? align_up((size_t)p.splits * s.uv * vec_size(dt), 256) : 0;
+  p.kind = K_COLS_PHASED;
+  p.pps = ceil_div(s.v * es, 16);
+  p.vec16 = (s.v * es) % 16 == 0 && aligned(A, 16);
+  p.G = w;
+  p.chunk = ceil_div(s.nk, splits);
+  p.splits = ceil_div(s.nk, p.chunk);
+  p.grid = dim3((unsigned)ceil_div(s.u * p.pps, w), (unsigned)p.splits);
+}
+
+// Few outputs (v > 1) over many rows: the widest block of pieces that the
+// outputs fill, the rows split over one wave of blocks (1000000x64 mode 0:
+// FP64 949 -> 115 us, FP32 684 -> 46, E4M3 831 -> 33; 8388608x128: FP32 1158
+// -> 610, BF16 2740 -> 375).
+static bool plan_phased_few(Plan& p, const Shape& s, tvc_dtype dt, const void* A, int sms) {
+  const int64_t pieces = s.u * ceil_div(s.v * (int64_t)elem_size(dt), 16);
+  if (pieces > 16 * sms || s.nk < 4096) return false;
+  int w = 1;
+  while (w < kThreads && w < pieces) w *= 2;
+  const int64_t blocks = (int64_t)sms * phased_blocks_per_sm(dt);
+  const int64_t splits = std::min(std::max<int64_t>(1, blocks / ceil_div(pieces, w)),
+                                  std::max<int64_t>(1, s.nk * w / (16 * kThreads)));
+  set_phased(p, s, dt, A, w, splits);
+  return true;
+}
+
+static void plan_cols_phased(Plan& p, const Shape& s, tvc_dtype dt, const void* A, int sms) {
+  if (plan_phased_few(p, s, dt, A, sms)) return;
+  const int64_t es = (int64_t)elem_size(dt), pieces = s.u * ceil_div(s.v * es, 16);
+  const int64_t blocks = (int64_t)sms * phased_blocks_per_sm(dt);
+  int64_t splits = 1;
+  int w = 8;
+  if (s.N * es <= kPhasedSmall && s.nk >= 8) {
+    w = 128;
+    while (w > 8 && ceil_div(pieces, w) < blocks) w /= 2;
+    while (s.nk * w < 4 * kThreads && w < 128) w *= 2;
+    if (ceil_div(pieces, w) < sms / 2)
+      splits = std::min(blocks / ceil_div(pieces, w), std::max<int64_t>(1, s.nk * w / (4 * kThreads)));
+  } else {
+    return;
+  }
+  set_phased(p, s, dt, A, w, splits);
+}
+
 static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool allow_staged) {
   Plan p;
   const bool f64acc = (dt == TVC_F64 || dt == TVC_F32D);  // FP64 arithmetic (float-float kernels)
@@ -1634,17 +1734,28 @@ static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool all
   const int64_t target_threads = (int64_t)sms * 2048;
   const int64_t S = s.nk * s.v;
   const size_t es = elem_size(dt);
-  const bool ragged = dt != TVC_F64 && dt != TVC_F32D && pick_vec(dt, s.v == 1 ? s.nk : s.v, A) * (int)es < 16;
+  // Rows off 16-byte boundaries (tvc_ragged.cu); FP32 columns only where the
+  // pieces give enough threads (64x264x475 mode 1: 8.5 us, element loads 7.5).
+  const bool ragged = dt != TVC_F64 && dt != TVC_F32D && pick_vec(dt, s.v == 1 ? s.nk : s.v, A) * (int)es < 16 &&
+                      !(dt == TVC_F32 && s.v >= 32 && s.u * ceil_div(s.v, 4) < (int64_t)sms * 64);
   if (s.v >= 32) {
     p.kind = ragged ? K_COLS_RAGGED : K_COLS;
     p.vec = pick_vec(dt, s.v, A);
     p.pps = ceil_div(s.v * (int64_t)es, 16);
     const int64_t threads = ragged ? s.u * p.pps : ceil_div(s.uv, p.vec);
     int64_t splits = 1;
-    if (threads < target_threads) splits = std::min(ceil_div(target_threads, threads), std::max<int64_t>(1, s.nk / 64));
+    // Rows per split: at least 64 for large E4M3 tensors (their partial sums
+    // are four times the codes; 95x582x214x28 mode 0 70 us, 95 with 32), else
+    // 32 (FP32 3188x6936 mode 0 22.6 -> 16.5 us, FP64 128^3 16 -> 10.5), 16
+    // for small tensors of ragged rows (fewer threads, fewer rows in flight).
+    const bool small = s.N * (int64_t)es <= (64 << 20);
+    const int64_t min_rows = (ragged && small && s.nk >= 128) ? 16 : (dt == TVC_E4M3 && !small) ? 64 : 32;
+    if (threads < target_threads)
+      splits = std::min(ceil_div(target_threads, threads), std::max<int64_t>(1, s.nk / min_rows));
     p.chunk = ceil_div(ceil_div(s.nk, splits), 8) * 8;
     p.splits = ceil_div(s.nk, p.chunk);
     p.grid = dim3((unsigned)ceil_div(threads, kThreads), (unsigned)p.splits);
+    plan_cols_phased(p, s, dt, A, sms);
   } else if (dt == TVC_F64 && aligned(A, 16) && s.v < 32 && plan_f64_tile(p, s, sms)) {
     // FP64 small slabs and short rows: the copy-engine tile kernel.
   } else if (s.v == 1 && !f64acc && ragged && rows_ragged_wanted(s.nk, es)) {
@@ -1757,6 +1868,8 @@ static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool all
     p.grid = dim3((unsigned)ceil_div(s.u, rows_per_block), (unsigned)p.splits);
   } else if (!f64acc && aligned(A, 16) && plan_slab_tile(p, s, dt, sms)) {
     // large slabs of whole 16-byte rows: the copy-engine slab kernel
+  } else if (plan_phased_few(p, s, dt, A, sms)) {
+    // few slabs of many rows: phases of rows over one wave of blocks
   } else if (S > 512 &&
              (dt == TVC_E4M3 || ((dt == TVC_BF16 || dt == TVC_F16) && s.v % 2 == 0) ||
               (dt == TVC_F32 && s.v % 4 == 0)) &&
@@ -1806,6 +1919,7 @@ static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool all
   if (f64acc) p.ws_xs = align_up((size_t)s.nk * sizeof(XSplit), 256);
   if (p.xs_shift) p.ws_xs += align_up((size_t)(s.nk + 2) * sizeof(XSplit), 256);
   if (p.splits > 1) p.ws_partial = align_up((size_t)p.splits * s.uv * vec_size(dt), 256);
+  p.ws_partial = std::max(p.ws_partial, p.ws_least);
   p.ws_total = p.ws_xs + p.ws_partial;
   return p;
 }
@@ -1951,6 +2065,9 @@ static bool launch_main(const Plan& p, const TvcArgs<DT>& a, cudaStream_t st) {
       }
       break;
     }
+    case K_COLS_PHASED:
+      cols_phased_launch<DT>(a, p.grid, p.pps, p.G, p.vec16 != 0, st);
+      break;
     case K_COLS_RAGGED:
       if constexpr (!kF64Acc<DT>) cols_ragged_launch<DT>(a, p.grid, p.pps, st);
       break;
@@ -2039,7 +2156,8 @@ static tvc_status run(const void* A, const Shape& s, const void* x, void* y, con
   a.vsh = -1;
   if (s.uv < ((int64_t)1 << 32) && s.v < ((int64_t)1 << 32)) div_magic((uint32_t)s.v, &a.vmag, &a.vsh);
   char* w = static_cast<char*>(ws);
-  if (kF64Acc<DT>) {
+  const bool split_x = kF64Acc<DT> && p.kind != K_COLS_PHASED;  // that kernel splits x itself
+  if (split_x) {
     a.xs = reinterpret_cast<const XSplit*>(w);
     XSplit* xs1 = p.xs_shift ? reinterpret_cast<XSplit*>(w + align_up((size_t)s.nk * sizeof(XSplit), 256)) : nullptr;
     a.xs1 = xs1;
@@ -2049,12 +2167,17 @@ static tvc_status run(const void* A, const Shape& s, const void* x, void* y, con
   }
   if (p.splits > 1) a.partial = w + p.ws_xs;
   if (!launch_main<DT>(p, a, st)) return TVC_ERR_UNSUPPORTED;
-  count_launches((kF64Acc<DT> ? 1 : 0) + 1 + (p.splits > 1 ? 1 : 0));
+  count_launches((split_x ? 1 : 0) + 1 + (p.splits > 1 ? 1 : 0));
   if (p.splits > 1) {
     using V = typename Elem<DT>::V;
-    const int blocks = (int)std::min<int64_t>(ceil_div(s.uv, 256), 8192);
-    tvc_reduce_kernel<V><<<blocks, 256, 0, st>>>(static_cast<const V*>(a.partial), static_cast<V*>(y), s.uv,
-                                                 p.splits, alpha, beta, done);
+    if (p.splits >= 32 && s.uv <= 32 * 1024) {
+      tvc_reduce_many_kernel<V><<<(int)ceil_div(s.uv, 32), 1024, 0, st>>>(
+          static_cast<const V*>(a.partial), static_cast<V*>(y), s.uv, p.splits, alpha, beta, done);
+    } else {
+      const int blocks = (int)std::min<int64_t>(ceil_div(s.uv, 256), 8192);
+      tvc_reduce_kernel<V><<<blocks, 256, 0, st>>>(static_cast<const V*>(a.partial), static_cast<V*>(y), s.uv,
+                                                   p.splits, alpha, beta, done);
+    }
   }
   return cuda_status(cudaGetLastError());
 }

@@ -166,4 +166,11 @@ void cols_ragged_launch(const TvcArgs<DT>& a, dim3 grid, int64_t pps, cudaStream
 template <tvc_dtype DT>
 void rows_ragged_launch(const TvcArgs<DT>& a, dim3 grid, int G, cudaStream_t st);
 
+// Few outputs (v > 1, tvc_phased.cu): blocks of w 16-byte pieces of the
+// outputs (a power of two up to 256, pps pieces per row) and 256 / w phases
+// of rows; al: every row starts on a 16-byte boundary.
+inline int phased_blocks_per_sm(tvc_dtype dt) { return dt == TVC_E4M3 ? 2 : 3; }  // resident at once
+template <tvc_dtype DT>
+void cols_phased_launch(const TvcArgs<DT>& a, dim3 grid, int64_t pps, int w, bool al, cudaStream_t st);
+
 }  // namespace tvcg
