@@ -8,157 +8,263 @@
 // gx, v == 1 and k > 0: gx = (A viewed as u x n_k) x_0 gy, i.e. a TVC of
 //   mode 0 on the unfolded view (the column kernel), with gy times the slab
 //   scale for narrow storage.
-// gx, otherwise: each thread owns VEC columns (i, l) of a column tile, keeps
-//   gy[i][l] in registers and accumulates A[i][j][l]*gy[i][l] into one
-//   register accumulator per row j of a chunk of JC rows; blocks walk the
-//   column tiles persistently, then reduce their accumulators (warp
-//   shuffles, then warps in a fixed order) to one partial row per block; a
-//   second kernel adds the blocks' partials in a fixed order.  A is read
-//   once; gy once per chunk of rows.
-// gA: threads own a position and loop over the other index so that every
-//   store is coalesced: columns (i, l) looping over j when v >= 32,
-//   positions q = (j, l) of a slab looping over slabs i otherwise.
+// gx, otherwise: each thread owns a 16-byte piece of columns (i, l), keeps
+//   its gy in registers and streams the piece's rows, eight (rows off 16-byte
+//   boundaries: four) in flight; a warp reduces the rows' dot products over
+//   its lanes with halving exchanges into its own sums of a chunk of rows in
+//   shared memory.  Blocks walk the pieces persistently and leave one partial
+//   row each; a second kernel adds the blocks' partials in a fixed order.  A
+//   is read once; gy once per chunk of rows.
+// gA: threads own 16 bytes (or one element where rows or slabs are not whole
+//   pieces) of columns (i, l), looping over j, when v >= 32, of positions (j,
+//   l) of a slab, looping over slabs i, below.
 #include <algorithm>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
+#include "ragged.cuh"
 
 namespace tvcg {
 
 constexpr int kBT = 256;  // threads per block
 constexpr int kBW = kBT / kWarp;
+constexpr int kGxRows = 256;  // rows per chunk at most
 
 template <tvc_dtype DT>
 struct GradArgs {
   const typename Elem<DT>::T* A;
   const void* gy;   // vector type (FP64 / FP32)
   const float* scales;
-  void* partial;    // [gridDim.x][nk] per chunk, vector type
-  int64_t u, nk, v, uv, upi0;
+  void* partial;    // [nblk][nk], vector type
+  int64_t u, nk, v, upi0, pps, nblk;
   int mode0;
-  int jc;           // rows per chunk (<= JC)
+  int rch;          // rows per chunk (<= kGxRows)
 };
 
 // ------------------------------------------------------------- gx, v >= 2
 
-template <tvc_dtype DT, int VEC, int JC>
-__global__ void __launch_bounds__(kBT) tvc_gradx_kernel(const GradArgs<DT> a) {
+// A 16-byte piece as the compute type.
+template <tvc_dtype DT>
+__device__ __forceinline__ void gx_piece(const uint4& w, typename Elem<DT>::C (&r)[16 / Elem<DT>::kSize]) {
+  if constexpr (DT == TVC_F64) {
+    r[0] = __hiloint2double((int)w.y, (int)w.x);
+    r[1] = __hiloint2double((int)w.w, (int)w.z);
+  } else if constexpr (DT == TVC_F32D) {
+    Elem<TVC_F32>::decode16(w, r);
+  } else {
+    Elem<DT>::decode16(w, r);
+  }
+}
+
+// The sums over the warp's lanes of a[0..M-1], the kept values halved per
+// exchange: lane L returns the sum of a[L / (32 / M)].
+template <int M>
+__device__ __forceinline__ float gx_lanes(float (&a)[M]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = M / 2, bit = 16; h >= 1; h >>= 1, bit >>= 1) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int e = 0; e < h; e++) {
+      const float mine = up ? a[e + h] : a[e], other = up ? a[e] : a[e + h];
+      a[e] = mine + __shfl_xor_sync(0xFFFFFFFFu, other, bit);
+    }
+  }
+  float r = a[0];
+#pragma unroll
+  for (int bit = 16 / M; bit >= 1; bit >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, bit);
+  return r;
+}
+
+// The same for float-float pairs (TwoSum per exchange).
+template <int M>
+__device__ __forceinline__ void gx_lanes(float (&s)[M], float (&c)[M]) {
+  const int lane = threadIdx.x & 31;
+  auto join = [](float& s0, float& c0, float s1, float c1) {
+    float t, err;
+    two_sum(s0, s1, t, err);
+    s0 = t;
+    c0 = __fadd_rn(__fadd_rn(c0, c1), err);
+  };
+#pragma unroll
+  for (int h = M / 2, bit = 16; h >= 1; h >>= 1, bit >>= 1) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int e = 0; e < h; e++) {
+      const float os = up ? s[e] : s[e + h], oc = up ? c[e] : c[e + h];
+      s[e] = up ? s[e + h] : s[e];
+      c[e] = up ? c[e + h] : c[e];
+      join(s[e], c[e], __shfl_xor_sync(0xFFFFFFFFu, os, bit), __shfl_xor_sync(0xFFFFFFFFu, oc, bit));
+    }
+  }
+#pragma unroll
+  for (int bit = 16 / M; bit >= 1; bit >>= 1)
+    join(s[0], c[0], __shfl_xor_sync(0xFFFFFFFFu, s[0], bit), __shfl_xor_sync(0xFFFFFFFFu, c[0], bit));
+}
+
+// Bound: HBM.  128^4 FP32, modes 0-2: 190 us and a reduction of 15 -> 163 and
+// 3 (7.0 TB/s; the kernel before held 16 rows' sums and loads in 168
+// registers, one block per SM); 17x52x68x18x31 FP64 mode 1 127 -> 79 us,
+// 12x93x44x11x82 FP32 mode 3 136 -> 62.  Resident blocks per SM (the grid is
+// one wave of them):
+template <tvc_dtype DT>
+inline constexpr int kGxBlocks = DT == TVC_E4M3 ? 2 : 3;
+
+// AL: every row of A starts on a 16-byte boundary.
+template <tvc_dtype DT, bool AL>
+__global__ void __launch_bounds__(kBT, kGxBlocks<DT>) tvc_gradx_kernel(const GradArgs<DT> a) {
   using E = Elem<DT>;
   using T = typename E::T;
   using V = typename E::V;
-  const int64_t j0 = (int64_t)blockIdx.y * a.jc;
-  const int jn = (int)min((int64_t)a.jc, a.nk - j0);
-  const int64_t ncol = a.uv / VEC;  // VEC divides v, hence uv
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ double red[kBW][JC];
-  if constexpr (kF64Acc<DT>) {
-    float s[JC], c[JC];
-    double d[JC];
+  constexpr bool F64 = kF64Acc<DT>;
+  constexpr int ES = E::kSize, VEC = 16 / ES, RB = AL ? 8 : 4;
+  using Sum = std::conditional_t<F64, double, float2>;  // float2: compensated pair
+  __shared__ Sum sums[kBW][kGxRows];
+  const int64_t b = blockIdx.x % a.nblk, j0 = blockIdx.x / a.nblk * a.rch;
+  const int jn = (int)min((int64_t)a.rch, a.nk - j0);
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  Sum* const mine = sums[warp];
+  for (int j = lane; j < jn; j += 32) mine[j] = Sum{};
+  __syncwarp();
+  const uint64_t sb = (uint64_t)a.v * ES;
+  const int64_t pieces = a.u * a.pps;
+  for (int64_t q0 = b * kBT; q0 < pieces; q0 += a.nblk * kBT) {
+    const int64_t q = q0 + t;
+    const bool ok = q < pieces;
+    const int64_t i = !ok ? 0 : (q >> 32) ? q / a.pps : (int64_t)((uint32_t)q / (uint32_t)a.pps);
+    const int64_t l = ok ? (q - i * a.pps) * VEC : 0;
+    const int nv = ok ? (int)min((int64_t)VEC, a.v - l) : 0, bytes = nv * ES;
+    const uint64_t ad0 = reinterpret_cast<uint64_t>(a.A) + (uint64_t)((i * a.nk + j0) * a.v + l) * ES;
+    const V* const gyp = static_cast<const V*>(a.gy) + i * a.v + l;
+    // gy of the piece (zero past the row): split pieces, or FP32 with the slab scale
+    XSplit gs[F64 ? VEC : 1];
+    float gf[F64 ? 1 : VEC];
+    if constexpr (F64) {
 #pragma unroll
-    for (int q = 0; q < JC; q++) {
-      s[q] = 0.0f;
-      c[q] = 0.0f;
-      d[q] = 0.0;
-    }
-    int cnt = 0;
-    for (int64_t col = (int64_t)blockIdx.x * kBT + threadIdx.x; col < ncol; col += (int64_t)gridDim.x * kBT) {
-      const int64_t o = col * VEC;
-      const int64_t i = o / a.v, l = o - i * a.v;
-      const double* gyp = static_cast<const double*>(a.gy) + o;
-      XSplit gs[VEC];
-      double gd[VEC];
-#pragma unroll
-      for (int e = 0; e < VEC; e++) {
-        gd[e] = __ldg(gyp + e);
-        gs[e] = split_x(gd[e]);
-      }
-      const T* p = a.A + (i * a.nk + j0) * a.v + l;
-      typename E::C r[JC][VEC];
-#pragma unroll
-      for (int q = 0; q < JC; q++)
-        if (q < jn) E::template load<VEC>(p + (int64_t)q * a.v, r[q]);
-#pragma unroll
-      for (int q = 0; q < JC; q++)
-        if (q < jn) {
-#pragma unroll
-          for (int e = 0; e < VEC; e++) df_mac(s[q], c[q], d[q], r[q][e], gyp + e, gs[e]);
-        }
-      if (++cnt == 32) {  // keep the float-float pairs short
-#pragma unroll
-        for (int q = 0; q < JC; q++) {
-          d[q] += (double)s[q];
-          d[q] += (double)c[q];
-          s[q] = 0.0f;
-          c[q] = 0.0f;
-        }
-        cnt = 0;
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < JC; q++) {
-      double t = (d[q] + (double)s[q]) + (double)c[q];
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, off);
-      if (lane == 0) red[warp][q] = t;
-    }
-  } else {
-    AccF32<JC> acc;
-    acc.init();
-    int cnt = 0;
-    for (int64_t col = (int64_t)blockIdx.x * kBT + threadIdx.x; col < ncol; col += (int64_t)gridDim.x * kBT) {
-      const int64_t o = col * VEC;
-      const int64_t i = o / a.v, l = o - i * a.v;
-      const float* gyp = static_cast<const float*>(a.gy) + o;
-      float g[VEC];
+      for (int e = 0; e < VEC; e++) gs[e] = e < nv ? split_x(__ldg(gyp + e)) : XSplit{0.0f, 0.0f};
+    } else {
       float sc = 1.0f;
       if constexpr (kNarrow<DT>) {
         if (!a.mode0 && a.scales) sc = __ldg(a.scales + i / a.upi0);
       }
 #pragma unroll
-      for (int e = 0; e < VEC; e++) g[e] = __fmul_rn(__ldg(gyp + e), sc);
-      const T* p = a.A + (i * a.nk + j0) * a.v + l;
-      float r[JC][VEC];
-#pragma unroll
-      for (int q = 0; q < JC; q++)
-        if (q < jn) E::template load<VEC>(p + (int64_t)q * a.v, r[q]);
-#pragma unroll
-      for (int q = 0; q < JC; q++)
-        if (q < jn) {
-#pragma unroll
-          for (int e = 0; e < VEC; e++) acc.a[q] = __fmaf_rn(r[q][e], g[e], acc.a[q]);
-        }
-      if (++cnt == 16) {
-        acc.fold();
-        cnt = 0;
-      }
+      for (int e = 0; e < VEC; e++) gf[e] = e < nv ? __fmul_rn(__ldg(gyp + e), sc) : 0.0f;
     }
-    acc.fold();
+    uint64_t ad = ad0;
+    for (int j = 0; j < jn; j += RB) {
+      Chunks ch[RB];
+      uint32_t sh[RB];
 #pragma unroll
-    for (int q = 0; q < JC; q++) {
-      float t = acc.result(q);
+      for (int e = 0; e < RB; e++) {
+        ch[e].a = ch[e].b = make_uint4(0u, 0u, 0u, 0u);
+        if (ok && j + e < jn) {
+          if constexpr (AL)
+            ch[e].a = __ldcs(reinterpret_cast<const uint4*>(ad));
+          else
+            ld_chunks(ad, bytes, ch[e]);
+        }
+        sh[e] = (uint32_t)ad & 15;
+        ad += sb;
+      }
+      if constexpr (F64) {
+        float s[RB], c[RB];
+        uint32_t bad = 0;
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, off);
-      if (lane == 0) red[warp][q] = (double)t;
+        for (int e = 0; e < RB; e++) {
+          typename E::C r[VEC];
+          gx_piece<DT>(AL ? ch[e].a : cut<ES>(ch[e], sh[e]), r);
+          s[e] = c[e] = 0.0f;
+          if (j + e < jn) {
+#pragma unroll
+            for (int x = 0; x < VEC; x++)
+              if (x < nv) df_step(s[e], c[e], bad, r[x], gs[x]);
+          }
+          bad |= isfinite(__fadd_rn(s[e], c[e])) ? 0u : 1u;
+        }
+        if (__any_sync(0xFFFFFFFFu, bad != 0)) {
+          // an element or an entry of gy outside the exact window: these
+          // rows again with FP64 multiply-adds
+          for (int e = 0; e < RB && j + e < jn; e++) {
+            double d = 0.0;
+            for (int x = 0; x < nv; x++)
+              d = fma((double)*reinterpret_cast<const T*>(ad0 + (uint64_t)(j + e) * sb + x * ES), __ldg(gyp + x), d);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, off);
+            if (lane == 0) mine[j + e] += d;
+          }
+          __syncwarp();
+        } else {
+          gx_lanes<RB>(s, c);
+          const int row = lane / (32 / RB);
+          if (lane % (32 / RB) == 0 && j + row < jn) mine[j + row] += (double)s[0] + (double)c[0];
+          __syncwarp();
+        }
+      } else {
+        float s[RB];
+#pragma unroll
+        for (int e = 0; e < RB; e++) {
+          float r[VEC];
+          gx_piece<DT>(AL ? ch[e].a : cut<ES>(ch[e], sh[e]), r);
+          if (nv < VEC) {  // what follows the row is another row
+#pragma unroll
+            for (int x = 0; x < VEC; x++) r[x] = x < nv ? r[x] : 0.0f;
+          }
+          s[e] = 0.0f;
+#pragma unroll
+          for (int x = 0; x < VEC; x++) s[e] = __fmaf_rn(r[x], gf[x], s[e]);
+        }
+        const float v = gx_lanes<RB>(s);
+        const int row = lane / (32 / RB);
+        if (lane % (32 / RB) == 0 && j + row < jn) {
+          const float2 o = mine[j + row];
+          float sum, err;
+          two_sum(o.x, v, sum, err);
+          mine[j + row] = make_float2(sum, __fadd_rn(o.y, err));
+        }
+        __syncwarp();
+      }
     }
   }
   __syncthreads();
-  if ((int)threadIdx.x < jn) {
-    const int q = threadIdx.x;
-    double t = 0.0;
-    for (int w = 0; w < kBW; w++) t += red[w][q];
-    V val = (V)t;
-    if constexpr (kNarrow<DT>) {
-      if (a.mode0 && a.scales) val = __fmul_rn(val, __ldg(a.scales + j0 + q));
+  for (int j = t; j < jn; j += kBT) {
+    V val;
+    if constexpr (F64) {
+      val = sums[0][j];
+      for (int w = 1; w < kBW; w++) val += sums[w][j];
+    } else {
+      KahanF32 k;
+      for (int w = 0; w < kBW; w++) {
+        k.add(sums[w][j].x);
+        k.add(sums[w][j].y);
+      }
+      val = k.value();
+      if constexpr (kNarrow<DT>) {
+        if (a.mode0 && a.scales) val = __fmul_rn(val, __ldg(a.scales + j0 + j));
+      }
     }
-    static_cast<V*>(a.partial)[(int64_t)blockIdx.x * a.nk + j0 + q] = val;
+    static_cast<V*>(a.partial)[b * a.nk + j0 + j] = val;
   }
 }
 
+// gx[j] = the blocks' partial sums in FP64, 32 entries per block: each warp a
+// contiguous share of the blocks in order, then the warps in order.
 template <class V>
-__global__ void tvc_gradx_reduce_kernel(const V* __restrict__ partial, V* __restrict__ gx, int64_t nk, int64_t nblk) {
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < nk; j += (int64_t)gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int64_t b = 0; b < nblk; b++) s += (double)partial[b * nk + j];
+__global__ void __launch_bounds__(kBT) tvc_gradx_reduce_kernel(const V* __restrict__ partial, V* __restrict__ gx,
+                                                              int64_t nk, int64_t nblk) {
+  __shared__ double sums[kBW][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t j = (int64_t)blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (j < nk) {
+#pragma unroll 8
+    for (int64_t b = nblk * w / kBW; b < nblk * (w + 1) / kBW; b++) s += (double)partial[b * nk + j];
+  }
+  sums[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && j < nk) {
+    for (int q = 1; q < kBW; q++) s += sums[q][lane];
     gx[j] = (V)s;
   }
 }
@@ -172,36 +278,78 @@ __global__ void tvc_scale_gy_kernel(const float* __restrict__ gy, const float* _
 
 // ------------------------------------------------------------------- gA
 
-template <class V>
-__global__ void tvc_gradA_cols_kernel(const V* __restrict__ gy, const V* __restrict__ x, V* __restrict__ gA,
-                                      int64_t uv, int64_t nk, int64_t v, double beta) {
-  // thread = column (i, l); loop over j
-  for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < uv; o += (int64_t)gridDim.x * blockDim.x) {
+// W products from p on in one store (W elements of 16 bytes, or one); BETA:
+// plus beta times what is there.
+template <class V, int W, bool BETA>
+__device__ __forceinline__ void gA_store(V* p, const V (&g)[W], const V (&x)[W], double beta) {
+  V val[W];
+#pragma unroll
+  for (int e = 0; e < W; e++) {
+    val[e] = g[e] * x[e];
+    if constexpr (BETA) val[e] += (V)beta * p[e];
+  }
+  if constexpr (W > 1) {
+    uint4 o;
+    memcpy(&o, val, 16);
+    __stcs(reinterpret_cast<uint4*>(p), o);
+  } else {
+    __stcs(p, val[0]);
+  }
+}
+
+// Bound: HBM writes (128^4 FP32 158-162 us in every mode; mode 3 412 with one
+// position per thread), FP64 the rate of its multiplications (33.5e6 elements
+// 139 -> 71 us with eight rows unrolled).
+// v >= 32: a thread owns W adjacent columns (i, l) and walks the rows j of
+// its part of n_k (blockIdx.y).  W > 1: v a multiple of W, gA 16-byte aligned.
+template <class V, int W, bool BETA>
+__global__ void __launch_bounds__(256) tvc_gradA_cols_kernel(const V* __restrict__ gy, const V* __restrict__ x,
+                                                             V* __restrict__ gA, int64_t uv, int64_t nk, int64_t v,
+                                                             int64_t chunk, double beta) {
+  const int64_t j0 = blockIdx.y * chunk, j1 = min(nk, j0 + chunk);
+  for (int64_t o = ((int64_t)blockIdx.x * 256 + threadIdx.x) * W; o < uv; o += (int64_t)gridDim.x * 256 * W) {
     const int64_t i = o / v, l = o - i * v;
-    const V g = gy[o];
-    V* p = gA + i * nk * v + l;
-    for (int64_t j = 0; j < nk; j++, p += v) {
-      V val = g * __ldg(x + j);
-      if (beta != 0.0) val += (V)beta * *p;
-      __stcs(p, val);
+    V g[W];
+#pragma unroll
+    for (int e = 0; e < W; e++) g[e] = __ldg(gy + o + e);
+    V* p = gA + (i * nk + j0) * v + l;
+#pragma unroll 8
+    for (int64_t j = j0; j < j1; j++, p += v) {
+      const V xj = __ldg(x + j);
+      V xs[W];
+#pragma unroll
+      for (int e = 0; e < W; e++) xs[e] = xj;
+      gA_store<V, W, BETA>(p, g, xs, beta);
     }
   }
 }
 
-template <class V>
-__global__ void tvc_gradA_slab_kernel(const V* __restrict__ gy, const V* __restrict__ x, V* __restrict__ gA,
-                                      int64_t u, int64_t nk, int64_t v, double beta) {
-  // thread = position q = j*v + l of a slab; loop over slabs i
+// v < 32: a thread owns W adjacent positions q = j*v + l of the slab (x_j in
+// registers) and walks the slabs; a block narrower than the slab's pieces
+// takes several slabs at once.  W > 1: the slab a multiple of W elements, gA
+// 16-byte aligned.
+template <class V, int W, bool BETA>
+__global__ void __launch_bounds__(256) tvc_gradA_slab_kernel(const V* __restrict__ gy, const V* __restrict__ x,
+                                                             V* __restrict__ gA, int64_t u, int64_t nk, int64_t v,
+                                                             int CW, double beta) {
   const int64_t S = nk * v;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < S; q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t j = q / v, l = q - j * v;
-    const V xj = x[j];
-    for (int64_t i = blockIdx.y; i < u; i += gridDim.y) {
-      V* p = gA + i * S + q;
-      V val = __ldg(gy + i * v + l) * xj;
-      if (beta != 0.0) val += (V)beta * *p;
-      __stcs(p, val);
-    }
+  const int P = 256 / CW, ph = threadIdx.x / CW;
+  const int64_t q = ((int64_t)blockIdx.x * CW + threadIdx.x - ph * CW) * W;
+  if (ph >= P || q >= S) return;
+  V xs[W];
+  int l[W];
+#pragma unroll
+  for (int e = 0; e < W; e++) {
+    const int64_t j = (q + e) / v;
+    xs[e] = __ldg(x + j);
+    l[e] = (int)(q + e - j * v);
+  }
+#pragma unroll 4
+  for (int64_t i = (int64_t)blockIdx.y * P + ph; i < u; i += (int64_t)gridDim.y * P) {
+    V g[W];
+#pragma unroll
+    for (int e = 0; e < W; e++) g[e] = __ldg(gy + i * v + l[e]);
+    gA_store<V, W, BETA>(gA + i * S + q, g, xs, beta);
   }
 }
 
@@ -211,8 +359,9 @@ namespace {
 
 struct GxPlan {
   bool via_tvc = false;  // v == 1
-  int vec = 1, jc = 8;
-  int64_t nchunks = 1, nblk = 1;
+  int rch = 8;        // rows per chunk
+  bool al = false;    // rows of A on 16-byte boundaries
+  int64_t nchunks = 1, nblk = 1, pps = 1;
   size_t ws_partial = 0, ws_gy = 0, ws_tvc = 0, total = 0;
   Shape view;  // v == 1: (u, nk) mode 0
 };
@@ -234,27 +383,20 @@ GxPlan plan_gx(const Shape& s, tvc_dtype dt, const void* A) {
     g.total = align_up(g.ws_tvc, 256) + g.ws_gy;
     return g;
   }
-  const int es = (int)elem_size(dt);
-  const int cand = (dt == TVC_F64) ? 2 : ((dt == TVC_F32) ? 4 : 4);
-  g.vec = 1;
-  if (s.v % cand == 0 && aligned(A, (size_t)cand * es)) g.vec = cand;
-  g.jc = (dt == TVC_F64 || dt == TVC_F32D) ? 8 : 16;
-  g.nchunks = cdiv(s.nk, g.jc);
-  const int64_t cols = s.uv / g.vec;
-  const int64_t want = std::max<int64_t>(1, (int64_t)device_sms() * 4 / std::max<int64_t>(1, g.nchunks));
-  g.nblk = std::max<int64_t>(1, std::min<int64_t>(cdiv(cols, kBT), want));
+  const int64_t es = (int64_t)elem_size(dt);
+  g.al = (s.v * es) % 16 == 0 && aligned(A, 16);
+  g.pps = cdiv(s.v * es, 16);
+  // One wave of blocks: chunks of 256 rows, or fewer (down to 32) where the
+  // pieces alone do not fill it.
+  const int64_t wave = (int64_t)device_sms() * (dt == TVC_E4M3 ? kGxBlocks<TVC_E4M3> : kGxBlocks<TVC_F32>);
+  const int64_t tiles = cdiv(s.u * g.pps, kBT);
+  g.nchunks = std::max(cdiv(s.nk, kGxRows), std::min(cdiv(s.nk, 32), wave / tiles));
+  g.rch = (int)(cdiv(cdiv(s.nk, g.nchunks), 8) * 8);
+  g.nchunks = cdiv(s.nk, g.rch);
+  g.nblk = std::max<int64_t>(1, std::min(tiles, wave / g.nchunks));
   g.ws_partial = align_up((size_t)g.nblk * s.nk * vs, 256);
   g.total = g.ws_partial;
   return g;
-}
-
-template <tvc_dtype DT, int VEC>
-void launch_gx(const GxPlan& g, const GradArgs<DT>& a, cudaStream_t st) {
-  dim3 grid((unsigned)g.nblk, (unsigned)g.nchunks);
-  if constexpr (kF64Acc<DT>)
-    tvc_gradx_kernel<DT, VEC, 8><<<grid, kBT, 0, st>>>(a);
-  else
-    tvc_gradx_kernel<DT, VEC, 16><<<grid, kBT, 0, st>>>(a);
 }
 
 template <tvc_dtype DT>
@@ -269,18 +411,17 @@ tvc_status run_gx(const GxPlan& g, const Shape& s, const void* A, const void* gy
   a.u = s.u;
   a.nk = s.nk;
   a.v = s.v;
-  a.uv = s.uv;
+  a.pps = g.pps;
+  a.nblk = g.nblk;
   a.upi0 = s.upi0 > 0 ? s.upi0 : 1;
   a.mode0 = s.mode == 0;
-  a.jc = g.jc;
-  if (g.vec == 1)
-    launch_gx<DT, 1>(g, a, st);
-  else if (g.vec == 2)
-    launch_gx<DT, 2>(g, a, st);
+  a.rch = g.rch;
+  const unsigned grid = (unsigned)(g.nblk * g.nchunks);
+  if (g.al)
+    tvc_gradx_kernel<DT, true><<<grid, kBT, 0, st>>>(a);
   else
-    launch_gx<DT, 4>(g, a, st);
-  const int blocks = (int)std::min<int64_t>(cdiv(s.nk, 256), 4096);
-  tvc_gradx_reduce_kernel<V><<<blocks, 256, 0, st>>>(static_cast<const V*>(ws), static_cast<V*>(gx), s.nk, g.nblk);
+    tvc_gradx_kernel<DT, false><<<grid, kBT, 0, st>>>(a);
+  tvc_gradx_reduce_kernel<V><<<(unsigned)cdiv(s.nk, 32), kBT, 0, st>>>(static_cast<const V*>(ws), static_cast<V*>(gx), s.nk, g.nblk);
   count_launches(2);
   return cuda_status(cudaGetLastError());
 }
@@ -314,18 +455,41 @@ tvc_status grad_x(const Shape& s, const void* A, const void* gy, void* gx, tvc_d
   return TVC_ERR_INVALID_ARG;
 }
 
+template <class V, int W, bool BETA>
+void launch_gA_w(const Shape& s, const V* x, const V* gy, V* gA, double beta, cudaStream_t st) {
+  const int64_t blocks = (int64_t)device_sms() * 16;
+  if (s.v >= 32) {
+    const int64_t bx = std::min<int64_t>(cdiv(s.uv, 256 * W), blocks);
+    const int64_t by = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cdiv(s.nk, 8), 65535), blocks / bx));
+    const int64_t chunk = cdiv(s.nk, by);
+    tvc_gradA_cols_kernel<V, W, BETA><<<dim3((unsigned)bx, (unsigned)cdiv(s.nk, chunk)), 256, 0, st>>>(
+        gy, x, gA, s.uv, s.nk, s.v, chunk, beta);
+  } else {
+    const int64_t pieces = s.nk * s.v / W;
+    const int CW = (int)std::min<int64_t>(pieces, 256);
+    const int64_t bx = cdiv(pieces, CW);
+    const int64_t by = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cdiv(s.u, 256 / CW), 65535), blocks / bx));
+    tvc_gradA_slab_kernel<V, W, BETA><<<dim3((unsigned)bx, (unsigned)by), 256, 0, st>>>(gy, x, gA, s.u, s.nk, s.v, CW,
+                                                                                       beta);
+  }
+}
+
+// Widest stores that the rows (v >= 32) or slabs (v < 32) allow.
+template <class V, bool BETA>
+void launch_gA(const Shape& s, const V* x, const V* gy, V* gA, double beta, cudaStream_t st) {
+  constexpr int W = 16 / (int)sizeof(V);
+  if (aligned(gA, 16) && (s.v >= 32 ? s.v : s.nk * s.v) % W == 0)
+    launch_gA_w<V, W, BETA>(s, x, gy, gA, beta, st);
+  else
+    launch_gA_w<V, 1, BETA>(s, x, gy, gA, beta, st);
+}
+
 template <class V>
 tvc_status grad_A(const Shape& s, const V* x, const V* gy, V* gA, double beta, cudaStream_t st) {
-  const int sms = device_sms();
-  if (s.v >= 32) {
-    const int blocks = (int)std::min<int64_t>(cdiv(s.uv, 256), (int64_t)sms * 16);
-    tvc_gradA_cols_kernel<V><<<blocks, 256, 0, st>>>(gy, x, gA, s.uv, s.nk, s.v, beta);
-  } else {
-    const int64_t S = s.nk * s.v;
-    const int64_t bx = std::min<int64_t>(cdiv(S, 256), (int64_t)sms * 16);
-    const int64_t by = std::max<int64_t>(1, std::min<int64_t>(s.u, std::min<int64_t>(65535, (int64_t)sms * 16 / bx + 1)));
-    tvc_gradA_slab_kernel<V><<<dim3((unsigned)bx, (unsigned)by), 256, 0, st>>>(gy, x, gA, s.u, s.nk, s.v, beta);
-  }
+  if (beta != 0.0)
+    launch_gA<V, true>(s, x, gy, gA, beta, st);
+  else
+    launch_gA<V, false>(s, x, gy, gA, beta, st);
   count_launches(1);
   return cuda_status(cudaGetLastError());
 }
