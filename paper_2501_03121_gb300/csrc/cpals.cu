@@ -34,21 +34,37 @@ struct KrArgs {
 
 // out = U_0 (.) U_1 (.) ... (.) U_{count-1} (columnwise Kronecker product,
 // row index with U_0's index most significant); count == 0 gives ones.
+// A thread computes up to four columns of one row, so the row's digits are
+// found once for them (16 x 2^20 transposed: 103 us with a thread per entry).
 template <class V>
 __global__ void khatri_rao_kernel(KrArgs a, V* __restrict__ out) {
-  const int64_t n = a.nrows * a.R;
+  const int64_t groups = (a.R + 3) / 4, n = a.nrows * groups;
+  const bool small = n <= 0xFFFFFFFFll;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t row = a.transposed ? e % a.nrows : e / a.R;
-    const int64_t r = a.transposed ? e / a.nrows : e % a.R;
-    V p = 1;
+    int64_t row, g;
+    if (a.transposed) {
+      g = small ? (int64_t)((uint32_t)e / (uint32_t)a.nrows) : e / a.nrows;
+      row = e - g * a.nrows;
+    } else {
+      row = small ? (int64_t)((uint32_t)e / (uint32_t)groups) : e / groups;
+      g = e - row * groups;
+    }
+    const int nr = (int)min((int64_t)4, a.R - 4 * g);
+    V p[4] = {1, 1, 1, 1};
     int64_t rem = row;
     for (int m = a.count - 1; m >= 0; m--) {
-      const int64_t im = rem % a.rows[m];
-      rem /= a.rows[m];
-      p *= static_cast<const V*>(a.U[m])[im * a.R + r];
+      const int64_t nm = a.rows[m];
+      const int64_t next = small ? (int64_t)((uint32_t)rem / (uint32_t)nm) : rem / nm;
+      const V* u = static_cast<const V*>(a.U[m]) + (rem - next * nm) * a.R + 4 * g;
+      rem = next;
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        if (q < nr) p[q] *= __ldg(u + q);
     }
-    if (a.scales) p *= (V)a.scales[row / a.per_slab];
-    out[e] = p;
+    const V sc = a.scales ? (V)a.scales[row / a.per_slab] : (V)1;
+#pragma unroll
+    for (int q = 0; q < 4; q++)
+      if (q < nr) out[a.transposed ? (4 * g + q) * a.nrows + row : row * a.R + 4 * g + q] = p[q] * sc;
   }
 }
 
@@ -93,15 +109,25 @@ __global__ void __launch_bounds__(kFinWarps * 32) mttkrp_finish_kernel(const V* 
       KahanF32 s;
       float blk = 0.0f;
       int c = 0;
-      for (int64_t q = w; q < K; q += kFinWarps) {
-        blk = __fmaf_rn(t[q1 * sq + q2 * sq2], W[q * R + r], blk);
-        q1 += d1;
-        q2 += d2;
-        if (q2 >= K2) {
-          q2 -= K2;
-          q1++;
+      for (int64_t q = w; q < K; q += 8 * kFinWarps) {
+        // eight terms in flight, folded every 64
+        float tv[8], wv[8];
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+          const bool in = q + e * kFinWarps < K;
+          tv[e] = in ? __ldg(t + q1 * sq + q2 * sq2) : 0.0f;
+          wv[e] = in ? __ldg(W + (q + e * kFinWarps) * R + r) : 0.0f;
+          q1 += d1;
+          q2 += d2;
+          if (q2 >= K2) {
+            q2 -= K2;
+            q1++;
+          }
         }
-        if (++c == 64) {
+#pragma unroll
+        for (int e = 0; e < 8; e++)
+          if (q + e * kFinWarps < K) blk = __fmaf_rn(tv[e], wv[e], blk);
+        if (++c == 8) {
           s.add(blk);
           blk = 0.0f;
           c = 0;
@@ -211,7 +237,7 @@ tvc_status kr_launch(const void* const* mats, const int64_t* rows, int count, in
   a.transposed = transposed;
   a.scales = scales;
   a.per_slab = per_slab > 0 ? per_slab : 1;
-  khatri_rao_kernel<V><<<grid_for(a.nrows * R), 256, 0, st>>>(a, static_cast<V*>(out));
+  khatri_rao_kernel<V><<<grid_for(a.nrows * ((R + 3) / 4)), 256, 0, st>>>(a, static_cast<V*>(out));
   count_launches(1);
   return cuda_status(cudaGetLastError());
 }

@@ -101,6 +101,26 @@ tvc_status tmc_tc_launch(const void* A, const Shape& s, const float* X, int64_t 
 // Sticky error word of that kernel's bounded waits (cleared when clear != 0).
 tvc_status tmc_tc_device_error(int* code_out, int clear);
 
+// Tensor-matrix contraction on the CUDA cores with register blocking
+// (tmc_simt.cu; FP32 accumulation, any alignment): rp rows of X per pass
+// (tmc_simt_rp), blocks_x = tmc_simt_blocks, n_k in `splits` chunks.
+struct TmcSimt {
+  const void* A = nullptr;
+  const float* X = nullptr;       // R x nk
+  const float* scales = nullptr;  // narrow types, nullable
+  float* Y = nullptr;             // u x R x v
+  float* partial = nullptr;       // splits x (u R v) when splits > 1
+  int64_t u = 0, nk = 0, v = 0, R = 0, upi0 = 1, chunk = 0, uRv = 0, blocks_x = 0;
+  int mode0 = 0, splits = 1, rp = 4, passes = 1, w = 256;  // w: tmc_simt_width (v > 1)
+  double alpha = 1.0, beta = 0.0;
+};
+int tmc_simt_rp(int64_t R);
+int tmc_simt_resident(int rp);  // blocks per SM
+int tmc_simt_width(int64_t u, int64_t v);
+int64_t tmc_simt_blocks(int64_t u, int64_t v);
+tvc_status tmc_simt_launch(const TmcSimt& a, tvc_dtype dt, cudaStream_t st);
+void tmc_simt_launch_narrow(const TmcSimt& a, tvc_dtype dt, bool al, cudaStream_t st);  // F16, E4M3
+
 // One pass over an R x C row-major matrix M (FP32, BF16, F16 or E4M3
 // storage) for T = M x (scaled per slab: T[r] *= scales[r / upi0] when
 // scales is given) and z = M^T w (dual.cu).  dual_supported says whether

@@ -654,16 +654,44 @@ __global__ void __launch_bounds__(kTmcThreads) tmc_rows_group_kernel(const TmcAr
   }
 }
 
-// Y[o] = alpha * sum_s partial[s][o] + beta * Y[o], s ascending.
+// Y[o] = alpha * sum_s partial[s][o] + beta * Y[o]: a block adds 32 outputs,
+// each of its 8 warps a contiguous share of the splits in order, then the
+// warps in order (FP32 compensated).
 template <class W>
-__global__ void tmc_reduce_kernel(const W* __restrict__ partial, W* __restrict__ Y, int64_t n, int splits,
-                                  double alpha, double beta) {
-  for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < n; o += (int64_t)gridDim.x * blockDim.x) {
-    W s = 0;
-    for (int k = 0; k < splits; k++) s += partial[(int64_t)k * n + o];
-    W r = (W)alpha * s;
-    if (beta != 0.0) r += (W)beta * Y[o];
-    Y[o] = r;
+__global__ void __launch_bounds__(256) tmc_reduce_kernel(const W* __restrict__ partial, W* __restrict__ Y, int64_t n,
+                                                         int splits, double alpha, double beta) {
+  __shared__ W sums[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  using Sum = std::conditional_t<sizeof(W) == 8, double, KahanF32>;
+  auto add = [](Sum& t, W v) {
+    if constexpr (sizeof(W) == 8)
+      t += v;
+    else
+      t.add(v);
+  };
+  auto value = [](const Sum& t) -> W {
+    if constexpr (sizeof(W) == 8)
+      return t;
+    else
+      return t.value();
+  };
+  for (int64_t o0 = (int64_t)blockIdx.x * 32; o0 < n; o0 += (int64_t)gridDim.x * 32) {
+    const int64_t o = o0 + lane;
+    Sum s{};
+    if (o < n) {
+#pragma unroll 8
+      for (int k = splits * w / 8; k < splits * (w + 1) / 8; k++) add(s, partial[(int64_t)k * n + o]);
+    }
+    __syncthreads();  // the previous outputs' sums are read
+    sums[w][lane] = value(s);
+    __syncthreads();
+    if (w == 0 && o < n) {
+      Sum t{};
+      for (int k = 0; k < 8; k++) add(t, sums[k][lane]);
+      W r = (W)alpha * value(t);
+      if (beta != 0.0) r += (W)beta * Y[o];
+      Y[o] = r;
+    }
   }
 }
 
@@ -676,6 +704,7 @@ struct TmcPlan {
   int64_t chunk = 0, blocks_x = 0;
   bool vj = false;
   bool tc = false;          // the tensor-core kernel (tmc_tc.cu)
+  bool simt = false;        // the register-blocked kernels (tmc_simt.cu)
   size_t ws = 0;
 };
 
@@ -684,6 +713,15 @@ int tmc_rp(tvc_dtype dt, int64_t R) {
   if (R <= 4) return 4;
   if (R <= 8 || f64) return 8;
   return 16;
+}
+
+// Whether the register-blocked kernels take the shape: FP32 accumulation,
+// where neither the copy pipelines for up to eight rows of X (p.async,
+// p.group) nor very short rows apply; columns against up to four rows of X
+// are bound by loads and stay with the one-element kernel (96x3935x409 FP32,
+// R = 4, mode 2 of the MTTKRP: 193 us, 214 here).
+bool simt_wanted(const TmcPlan& p, const Shape& s, tvc_dtype dt, int64_t R) {
+  return vec_size(dt) == 4 && !p.async && !p.group && (s.v == 1 ? s.nk >= 4 : s.v >= 4 && R > 4);
 }
 
 // A == nullptr (the workspace query) plans for a 16-byte aligned A; the
@@ -716,6 +754,20 @@ TmcPlan tmc_plan(const Shape& s, int64_t R, tvc_dtype dt, const void* A, bool a1
     p.group = g;
     const int64_t rpb = (kTmcThreads / 32) * (32 / g);
     p.blocks_x = (s.u + rpb - 1) / rpb;
+  }
+  if (simt_wanted(p, s, dt, R)) {
+    p.simt = true;
+    p.rp = tmc_simt_rp(R);
+    p.passes = (int)((R + p.rp - 1) / p.rp);
+    p.blocks_x = tmc_simt_blocks(s.u, s.v);
+    // one wave of resident blocks, at least 256 rows each
+    const int64_t have = p.blocks_x * p.passes, want = (int64_t)tmc_simt_resident(p.rp) * device_sms();
+    int64_t splits = 1;
+    if (have < want) splits = std::min<int64_t>(std::max<int64_t>(1, want / have), std::max<int64_t>(1, s.nk / 256));
+    p.chunk = ((s.nk + splits - 1) / splits + 63) / 64 * 64;
+    p.splits = (int)((s.nk + p.chunk - 1) / p.chunk);
+    p.ws = p.splits > 1 ? (size_t)p.splits * (size_t)(s.uv * R) * vec_size(dt) : 0;
+    return p;
   }
   const int64_t want = 4LL * device_sms();  // blocks for a full GPU
   int64_t have = p.blocks_x * p.passes;
@@ -805,7 +857,34 @@ tvc_status run(const void* A, const Shape& s, const void* X, int64_t R, void* Y,
   a.alpha = alpha;
   a.beta = beta;
   if (p.blocks_x > 0x7FFFFFFF || p.passes > 65535) return TVC_ERR_UNSUPPORTED;
-  switch (p.rp) {
+  if constexpr (!kF64Acc<DT>) {
+    if (p.simt) {
+      TmcSimt t;
+      t.A = A;
+      t.X = a.X;
+      t.scales = scales;
+      t.Y = a.Y;
+      t.partial = a.partial;
+      t.u = s.u;
+      t.nk = s.nk;
+      t.v = s.v;
+      t.R = R;
+      t.upi0 = s.upi0;
+      t.chunk = p.chunk;
+      t.uRv = a.uRv;
+      t.blocks_x = p.blocks_x;
+      t.mode0 = a.mode0;
+      t.splits = p.splits;
+      t.rp = p.rp;
+      t.passes = p.passes;
+      if (s.v > 1) t.w = tmc_simt_width(s.u, s.v);
+      t.alpha = alpha;
+      t.beta = beta;
+      const tvc_status rc = tmc_simt_launch(t, DT, st);
+      if (rc != TVC_OK) return rc;
+    }
+  }
+  if (!p.simt) switch (p.rp) {
     case 4: launch_rp<DT, 4>(a, p, st); break;
     case 8: launch_rp<DT, 8>(a, p, st); break;
     default:
@@ -815,7 +894,7 @@ tvc_status run(const void* A, const Shape& s, const void* X, int64_t R, void* Y,
   int launches = 1;
   if (p.splits > 1) {
     const int64_t n = s.uv * R;
-    const int blocks = (int)std::min<int64_t>((n + 255) / 256, 8LL * device_sms());
+    const int blocks = (int)std::min<int64_t>((n + 31) / 32, 64LL * device_sms());
     tmc_reduce_kernel<W><<<blocks, 256, 0, st>>>(static_cast<const W*>(ws), static_cast<W*>(Y), n, p.splits, alpha,
                                                  beta);
     launches++;
