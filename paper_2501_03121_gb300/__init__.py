@@ -168,13 +168,16 @@ def _dims_array(shape):
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    """Address of a tensor for a void* argument (None: NULL)."""
+    return t.data_ptr() if t is not None else None
 
 
 def _stream(stream):
+    """Handle of `stream`, or of the current device's current stream (asked
+    for by number: a Stream object per call costs more than a launch)."""
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _check(status, where):
