@@ -1754,6 +1754,10 @@ static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool all
     const int64_t min_rows = (ragged && small && s.nk >= 128) ? 16 : (dt == TVC_E4M3 && !small) ? 64 : 32;
     if (threads < target_threads)
       splits = std::min(ceil_div(target_threads, threads), std::max<int64_t>(1, s.nk / min_rows));
+    // A piece of up to 16 outputs per thread: the partial sums stay within the
+    // fixed scratch of tvc_noalloc, which takes these shapes (at two splits
+    // E4M3 2680x212x1690 mode 1 would need 36 MB).
+    if (ragged) splits = std::min(splits, std::max<int64_t>(1, TVC_NOALLOC_SCRATCH_BYTES / (s.uv * 4)));
     p.chunk = ceil_div(ceil_div(s.nk, splits), 8) * 8;
     p.splits = ceil_div(s.nk, p.chunk);
     p.grid = dim3((unsigned)ceil_div(threads, kThreads), (unsigned)p.splits);
