@@ -114,6 +114,11 @@ tvc_status stream_scratch_alloc(size_t bytes, cudaStream_t st, void** out) {
   return TVC_OK;
 }
 
+tvc_status stream_scratch_ready() {
+  cudaMemPool_t pool = nullptr;
+  return device_pool(&pool);
+}
+
 tvc_status stream_scratch_free(void* p, cudaStream_t st) {
   if (p == nullptr) return TVC_OK;
   return cuda_status(cudaFreeAsync(p, st));

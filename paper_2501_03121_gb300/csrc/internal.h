@@ -39,6 +39,7 @@ inline bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 // becomes the graph's own allocation and free nodes.  bytes == 0 gives NULL.
 tvc_status stream_scratch_alloc(size_t bytes, cudaStream_t st, void** out);
 tvc_status stream_scratch_free(void* p, cudaStream_t st);
+tvc_status stream_scratch_ready();  // creates the current device's pool if it is not there yet
 
 // cuTensorMapEncodeTiled, looked up once through the runtime (no link to the
 // driver library); NULL when the driver does not offer it.

@@ -2278,8 +2278,10 @@ extern "C" tvc_status tvc(const void* A, int order, const int64_t* dims, int mod
   void* ws = nullptr;
   if (uses_workspace(p, dtype)) {
     st = stream_scratch_alloc(p.ws_total, cs, &ws);
-    if (st != TVC_OK) return st;
+  } else if (p.ws_total > 0) {
+    st = stream_scratch_ready();  // as if it had allocated: a later captured call finds the pool
   }
+  if (st != TVC_OK) return st;
   st = launch_plan(A, s, x, y, dtype, nullptr, 1.0, 0.0, ws, p, cs, nullptr);
   const tvc_status fr = stream_scratch_free(ws, cs);
   return st != TVC_OK ? st : fr;
