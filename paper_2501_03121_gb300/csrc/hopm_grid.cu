@@ -438,7 +438,10 @@ __global__ void __launch_bounds__(kHgT, 1) hopm_grid_kernel(const HgArgs a) {
       }
       if (j > 0) src = W;
       want += (unsigned)B;
-      if (!grid_barrier(a.arrived, want, &s.flag)) return;
+      if (!grid_barrier(a.arrived, want, &s.flag)) {  // results invalid, as the error word says
+        if (b == 0 && t == 0 && a.status_out) *a.status_out = TVC_ERR_TIMEOUT;
+        return;
+      }
       // z_j from the parts, its norm and x_j, in every block alike
       auto entry = [&](int i) {
         if (last) return __ldcg(part + i);
