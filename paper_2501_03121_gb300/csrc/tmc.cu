@@ -18,6 +18,8 @@
 //     the RP partial sums are reduced over the lanes by a butterfly;
 //   * tmc_f64_kernel (FP64, single-double): float-float products on the
 //     FP32 pipe, FP64 totals;
+//   * tmc_simt.cuh: register-blocked kernels for FP32 accumulation at any
+//     alignment, where none of the above applies;
 //   * tmc_kernel: every other case, one output column per thread, 16 (8)
 //     rows in flight.
 // Few outputs split n_k over blockIdx.y; tmc_reduce_kernel adds the partial
@@ -721,7 +723,8 @@ int tmc_rp(tvc_dtype dt, int64_t R) {
 // are bound by loads and stay with the one-element kernel (96x3935x409 FP32,
 // R = 4, mode 2 of the MTTKRP: 193 us, 214 here).
 bool simt_wanted(const TmcPlan& p, const Shape& s, tvc_dtype dt, int64_t R) {
-  return vec_size(dt) == 4 && !p.async && !p.group && (s.v == 1 ? s.nk >= 4 : s.v >= 4 && R > 4);
+  return vec_size(dt) == 4 && !p.async && !p.group && (s.v == 1 ? s.nk >= 4 : s.v >= 4 && R > 4) &&
+         tmc_simt_blocks(s.u, s.v) * ((R + 3) / 4) <= 0x7FFFFFFF;  // one grid dimension
 }
 
 // A == nullptr (the workspace query) plans for a 16-byte aligned A; the
