@@ -343,8 +343,9 @@ size_t hopm_backward_workspace_size(int order, const int64_t* dims, tvc_dtype dt
  * Many independent FP32 tensors of any order and shape in one persistent
  * launch (the paper's task-based overlap of many contractions, Section
  * 4.3, done as a device work queue): one descriptor per tensor; the work is
- * cut into items of about 2^20 elements (output ranges of the contraction,
- * row ranges of gx, slab/row rectangles of gA), largest tensors first, and
+ * cut into items of 2^15 .. 2^19 elements (ranges of columns or rows for which
+ * y, gx and gA are formed from one read of A where the shape allows, else one
+ * item kind per result), largest tensors first, and
  * pulled by persistent blocks from an atomic counter.  (hopm_batched runs
  * one thread-block cluster per tensor.)
  * All pointers in a descriptor are device pointers, FP32, dense row-major.
