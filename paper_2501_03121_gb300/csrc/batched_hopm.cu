@@ -21,10 +21,11 @@
 // Bound: the two passes over A, latency (bytes in flight per SM) before HBM:
 // 512 threads of 64 registers, two blocks per SM, hold 64-128 bytes of A per
 // thread in flight.  512 tensors of 8..192 per mode (2.1e9 elements), 10
-// sweeps: 34.6 ms = 5.0 TB/s of the passes, 283 tensors 22 ms, 73 tensors and
-// 5 sweeps 4.2 ms; 4096 tensors 265 ms.  One block per tensor, the layout
-// before this one, took 109, 105, 52 and 287 ms: a single block streams about
-// 10 GB/s, and the launch ended with the largest tensors alone on the GPU.
+// sweeps: 32.8 ms = 5.2 TB/s of the passes, 283 tensors 22 ms, 73 tensors and
+// 5 sweeps 4.2 ms; 4096 tensors 265 ms (of another draw 305).  One block per
+// tensor, the layout before this one, took 117, 105, 52 and 287 ms (307): a
+// single block streams about 10 GB/s, and the launch ended with the largest
+// tensors alone on the GPU.
 // Streaming (evict-first) loads measured 5-8% faster than plain ones; 256
 // threads per block, or three blocks per SM, slower.
 #include <algorithm>
