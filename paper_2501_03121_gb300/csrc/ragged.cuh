@@ -13,11 +13,13 @@ struct Chunks {
 };
 
 // The aligned chunks that hold bytes [ad, ad + bytes), 1 <= bytes <= 16.
+// KEEP: ordinary loads instead of evict-first ones (the callers say why).
+template <bool KEEP = false>
 __device__ __forceinline__ void ld_chunks(uint64_t ad, int bytes, Chunks& c) {
   const uint4* p = reinterpret_cast<const uint4*>(ad & ~(uint64_t)15);
-  c.a = __ldcs(p);
+  c.a = KEEP ? __ldg(p) : __ldcs(p);
   c.b = make_uint4(0u, 0u, 0u, 0u);
-  if ((int)(ad & 15) + bytes > 16) c.b = __ldcs(p + 1);
+  if ((int)(ad & 15) + bytes > 16) c.b = KEEP ? __ldg(p + 1) : __ldcs(p + 1);
 }
 
 // The 16 bytes that start k = ad & 15 bytes into the chunks (ES: element

@@ -129,6 +129,11 @@ __global__ void __launch_bounds__(kRgThreads, kRgBlocks<DT>) tvc_cols_ragged_ker
 // 2541; of 331 4032 -> 5096, 1612 -> 4081, 929 -> 2944; of 979 4529 -> 5547,
 // 2118 -> 4574, 1343 -> 3265.  Three resident blocks (E4M3: 98 -> 80
 // registers): rows of 979 E4M3 2849 -> 3265.
+// Ordinary loads but for E4M3: a row's last chunk is the next row's first, and
+// a neighbouring group may reach it when an evict-first line is gone (rows of
+// 63 FP32 854 -> 787 us on 4.0 GB; every mode of 63^5 in turn 3313 -> 3165, of
+// BF16 175^4 1402 -> 1349, of E4M3 979^3 675 -> 681).  The columns, 3-10% slower
+// with them, keep evict-first (F16 972980x347 mode 0 230 against 252 us).
 template <tvc_dtype DT>
 __global__ void __launch_bounds__(kRgThreads, 3) tvc_rows_ragged_kernel(const TvcArgs<DT> a, int G) {
   if (skip(a.done)) return;
@@ -159,7 +164,7 @@ __global__ void __launch_bounds__(kRgThreads, 3) tvc_rows_ragged_kernel(const Tv
 #pragma unroll
     for (int b = 0; b < RB; b++) {
       c[b].a = c[b].b = make_uint4(0u, 0u, 0u, 0u);
-      if (row0 + b * gw < a.u) ld_chunks(base + b * gw * rb + (uint64_t)j * ES, nv * ES, c[b]);
+      if (row0 + b * gw < a.u) ld_chunks<DT != TVC_E4M3>(base + b * gw * rb + (uint64_t)j * ES, nv * ES, c[b]);
     }
     float xq[VEC];
     if (nv == VEC) {
