@@ -656,9 +656,13 @@ class TVCBatch:
 
 
 class HOPMBatch:
-    """A batch of FP32 power methods (one thread-block cluster per tensor, `iters` sweeps)."""
+    """A batch of FP32 power methods (one thread-block cluster per tensor, `iters` sweeps).
+    items: dicts with A (float32 CUDA tensor), x (its start vectors, updated
+    in place) and any of lam, status; the batch holds on to them, since the
+    uploaded descriptors keep their addresses."""
 
     def __init__(self, items, iters):
+        self.items = [{**it, "x": list(it["x"])} for it in items]
         self.iters = int(iters)
         n = len(items)
         arr = (_HopmBatchDesc * max(1, n))()
