@@ -236,8 +236,9 @@ __global__ void __launch_bounds__(kBT, kGxBlocks<DT>) tvc_gradx_kernel(const Gra
     } else {
       KahanF32 k;
       for (int w = 0; w < kBW; w++) {
-        k.add(sums[w][j].x);
-        k.add(sums[w][j].y);
+        const float2 o = sums[w][j];
+        k.add(o.x);
+        k.add(o.y == o.y ? o.y : 0.0f);  // NaN: o.x alone (see pair_value)
       }
       val = k.value();
       if constexpr (kNarrow<DT>) {

@@ -481,6 +481,11 @@ __device__ __forceinline__ void df_add_double(float& s, float& c, double d) {
   c = __fadd_rn(c, __fadd_rn(err, lo));
 }
 
+// The sum of a compensated pair.  TwoSum of an infinity (an infinite term, or
+// a sum beyond the largest binary32) leaves a NaN in c; s is then what plain
+// addition gives: the infinity, or NaN where infinities cancel.
+__device__ __forceinline__ float pair_value(float s, float c) { return c == c ? __fadd_rn(s, c) : s; }
+
 // ------------------------------------------------------------ accumulators
 
 // FP64 accumulator for VEC columns: float-float pairs plus an FP64 total.
@@ -550,7 +555,7 @@ struct AccF32 {
       a[e] = 0.0f;
     }
   }
-  __device__ __forceinline__ float result(int e) const { return __fadd_rn(S[e], C[e]); }
+  __device__ __forceinline__ float result(int e) const { return pair_value(S[e], C[e]); }
 };
 
 // Compensated FP32 sum helper for reductions of partial results.
@@ -562,7 +567,7 @@ struct KahanF32 {
     S = t;
     C = __fadd_rn(C, err);
   }
-  __device__ __forceinline__ float value() const { return __fadd_rn(S, C); }
+  __device__ __forceinline__ float value() const { return pair_value(S, C); }
 };
 
 }  // namespace tvcg

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kDualThreads) dual_kernel(const DualArgs a) {
       for (int k = 0; k < K; k++) {
         const int64_t c = (int64_t)(cw + WG * k) * CH + lane * VEC;
 #pragma unroll
-        for (int e = 0; e < VEC; e++) zsm[c + e] = __fadd_rn(zsm[c + e], __fadd_rn(zS[k][e], zC[k][e]));
+        for (int e = 0; e < VEC; e++) zsm[c + e] = __fadd_rn(zsm[c + e], pair_value(zS[k][e], zC[k][e]));
       }
     }
     __syncthreads();

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kRgThreads, kRgBlocks<DT>) tvc_cols_ragged_ker
   for (int e = 0; e < VEC; e++)
     if (e < nv) {
       const float2 t = my[e * kRgThreads];
-      emit(a, blockIdx.y, o + e, __fmul_rn(__fadd_rn(t.x, t.y), sc));
+      emit(a, blockIdx.y, o + e, __fmul_rn(pair_value(t.x, t.y), sc));
     }
 }
 

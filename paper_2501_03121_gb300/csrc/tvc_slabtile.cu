@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kStThreads, 2) tvc_slabtile_kernel(const TvcAr
     // warps in order
 #pragma unroll
     for (int e = 0; e < EPC; e++) {
-      float r = __fadd_rn(S[e], C[e]);
+      float r = pair_value(S[e], C[e]);
       for (int m = CPR; m < kWarp; m <<= 1) r = __fadd_rn(r, __shfl_xor_sync(0xFFFFFFFFu, r, m));
       if (lane < CPR) part[warp * v + lane * EPC + e] = r;
     }
