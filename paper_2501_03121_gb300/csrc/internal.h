@@ -120,7 +120,7 @@ int tmc_simt_resident(int rp);  // blocks per SM
 int tmc_simt_width(int64_t u, int64_t v);
 int64_t tmc_simt_blocks(int64_t u, int64_t v);
 tvc_status tmc_simt_launch(const TmcSimt& a, tvc_dtype dt, cudaStream_t st);
-void tmc_simt_launch_narrow(const TmcSimt& a, tvc_dtype dt, bool al, cudaStream_t st);  // F16, E4M3
+tvc_status tmc_simt_launch_narrow(const TmcSimt& a, tvc_dtype dt, bool al, cudaStream_t st);  // F16, E4M3
 
 // One pass over an R x C row-major matrix M (FP32, BF16, F16 or E4M3
 // storage) for T = M x (scaled per slab: T[r] *= scales[r / upi0] when

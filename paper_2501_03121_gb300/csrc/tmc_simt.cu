@@ -29,13 +29,12 @@ tvc_status tmc_simt_launch(const TmcSimt& a, tvc_dtype dt, cudaStream_t st) {
   const int64_t es = (int64_t)elem_size(dt), bytes = 4 * es;  // of a window
   const bool al = ((a.v == 1 ? a.nk : a.v) * es) % bytes == 0 && aligned(a.A, (size_t)bytes);
   switch (dt) {
-    case TVC_F32: launch_dt<TVC_F32>(a, al, st); break;
-    case TVC_BF16: launch_dt<TVC_BF16>(a, al, st); break;
+    case TVC_F32: return launch_dt<TVC_F32>(a, al, st);
+    case TVC_BF16: return launch_dt<TVC_BF16>(a, al, st);
     case TVC_F16:
-    case TVC_E4M3: tmc_simt_launch_narrow(a, dt, al, st); break;
+    case TVC_E4M3: return tmc_simt_launch_narrow(a, dt, al, st);
     default: return TVC_ERR_INVALID_ARG;
   }
-  return cuda_status(cudaGetLastError());
 }
 
 }  // namespace tvcg

@@ -25,6 +25,8 @@
 #pragma once
 
 #include <algorithm>
+#include <mutex>
+#include <set>
 #include <type_traits>
 
 #include "common.cuh"
@@ -465,15 +467,29 @@ __global__ void __launch_bounds__(kTsT, ts_blocks(RP)) tmc_rows_simt_kernel(cons
 
 // ------------------------------------------------------------------ host --
 
-template <class K>
-void smem_limit(K kern, size_t bytes) {
-  // cheap and idempotent; the attribute belongs to the device in use
-  if (bytes > 48 * 1024)
-    cudaFuncSetAttribute(reinterpret_cast<const void*>(kern), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+// Most shared memory a launch with RP rows of X asks for: columns with several
+// folds or phases (ts_stage_rows(P) * P <= 256 rows per stage of X).
+template <int RP>
+inline constexpr int kTsSmemMax = (256 * (RP + 4) + RP * 4 * kTsT) * (int)sizeof(float);
+
+// Opts a kernel in to `bytes` of dynamic shared memory, once per kernel and
+// device: the attribute belongs to the kernel, so a limit per launch would let
+// one host thread lower what another is about to launch with.
+inline cudaError_t smem_limit(const void* kern, int bytes) {
+  static std::mutex mu;
+  static std::set<std::pair<int, const void*>> done;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  if (done.count({dev, kern})) return cudaSuccess;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done.insert({dev, kern});
+  return e;
 }
 
 template <tvc_dtype DT, int RP>
-void launch_rp(const TmcSimt& a, bool al, cudaStream_t st) {
+tvc_status launch_rp(const TmcSimt& a, bool al, cudaStream_t st) {
   const dim3 grid((unsigned)(a.blocks_x * a.passes), (unsigned)a.splits);
   size_t smem;
   void (*kern)(const TmcSimt);
@@ -486,19 +502,21 @@ void launch_rp(const TmcSimt& a, bool al, cudaStream_t st) {
     if constexpr (RP > 4)
       kern = al ? tmc_cols_simt_kernel<DT, RP, true> : tmc_cols_simt_kernel<DT, RP, false>;
     else
-      return;  // columns against up to four rows of X stay with tmc.cu
+      return TVC_ERR_UNSUPPORTED;  // columns against up to four rows of X stay with tmc.cu
   }
-  smem_limit(kern, smem);
+  const cudaError_t e = smem_limit(reinterpret_cast<const void*>(kern), kTsSmemMax<RP>);
+  if (e != cudaSuccess) return cuda_status(e);
   kern<<<grid, kTsT, smem, st>>>(a);
+  return cuda_status(cudaGetLastError());
 }
 
 template <tvc_dtype DT>
-void launch_dt(const TmcSimt& a, bool al, cudaStream_t st) {
+tvc_status launch_dt(const TmcSimt& a, bool al, cudaStream_t st) {
   switch (a.rp) {
-    case 4: launch_rp<DT, 4>(a, al, st); break;
-    case 8: launch_rp<DT, 8>(a, al, st); break;
-    case 12: launch_rp<DT, 12>(a, al, st); break;
-    default: launch_rp<DT, 16>(a, al, st); break;
+    case 4: return launch_rp<DT, 4>(a, al, st);
+    case 8: return launch_rp<DT, 8>(a, al, st);
+    case 12: return launch_rp<DT, 12>(a, al, st);
+    default: return launch_rp<DT, 16>(a, al, st);
   }
 }
 

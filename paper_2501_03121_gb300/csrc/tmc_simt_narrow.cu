@@ -4,11 +4,8 @@
 
 namespace tvcg {
 
-void tmc_simt_launch_narrow(const TmcSimt& a, tvc_dtype dt, bool al, cudaStream_t st) {
-  if (dt == TVC_F16)
-    launch_dt<TVC_F16>(a, al, st);
-  else
-    launch_dt<TVC_E4M3>(a, al, st);
+tvc_status tmc_simt_launch_narrow(const TmcSimt& a, tvc_dtype dt, bool al, cudaStream_t st) {
+  return dt == TVC_F16 ? launch_dt<TVC_F16>(a, al, st) : launch_dt<TVC_E4M3>(a, al, st);
 }
 
 }  // namespace tvcg
