@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kBT, kGxBlocks<DT>) tvc_gradx_kernel(const Gra
   for (int64_t q0 = b * kBT; q0 < pieces; q0 += a.nblk * kBT) {
     const int64_t q = q0 + t;
     const bool ok = q < pieces;
-    const int64_t i = !ok ? 0 : (q >> 32) ? q / a.pps : (int64_t)((uint32_t)q / (uint32_t)a.pps);
+    const int64_t i = ok ? piece_row(q, a.pps) : 0;
     const int64_t l = ok ? (q - i * a.pps) * VEC : 0;
     const int nv = ok ? (int)min((int64_t)VEC, a.v - l) : 0, bytes = nv * ES;
     const uint64_t ad0 = reinterpret_cast<uint64_t>(a.A) + (uint64_t)((i * a.nk + j0) * a.v + l) * ES;

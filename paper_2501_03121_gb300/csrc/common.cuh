@@ -26,6 +26,7 @@
 #include <stdint.h>
 
 #include "../../include/tvc.h"
+#include "index.h"
 
 namespace tvcg {
 

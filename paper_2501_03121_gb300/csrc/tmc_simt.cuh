@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kTsT, ts_blocks(RP)) tmc_cols_simt_kernel(cons
   const int64_t r0 = (int64_t)(blockIdx.x - tile * a.passes) * RP;
   const int64_t ppr = (a.v + C - 1) / C, q = tile * w + ll;
   const bool act = ph < P && q < a.u * ppr;
-  const int64_t i = !act ? 0 : (q >> 32) ? q / ppr : (int64_t)((uint32_t)q / (uint32_t)ppr);
+  const int64_t i = act ? piece_row(q, ppr) : 0;
   const int64_t l = act ? (q - i * ppr) * C : 0;
   const int nv = act ? (int)min((int64_t)C, a.v - l) : 0;
   const int64_t j0 = (int64_t)blockIdx.y * a.chunk, j1 = min(a.nk, j0 + a.chunk);

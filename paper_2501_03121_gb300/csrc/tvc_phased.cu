@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kPhT, DT == TVC_E4M3 ? 2 : 3) tvc_cols_phased_
   const int t = threadIdx.x, P = kPhT / w, ph = t / w, ll = t - ph * w;
   const int64_t q = (int64_t)blockIdx.x * w + ll;
   const bool ok = q < a.u * pps;
-  const int64_t i = !ok ? 0 : (q >> 32) ? q / pps : (int64_t)((uint32_t)q / (uint32_t)pps);
+  const int64_t i = ok ? piece_row(q, pps) : 0;
   const int64_t l = ok ? (q - i * pps) * VEC : 0;
   const int nv = (int)min((int64_t)VEC, a.v - l), bytes = nv * ES;
   const int64_t jb = (int64_t)blockIdx.y * a.chunk, je = min(a.nk, jb + a.chunk);
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kPhT, DT == TVC_E4M3 ? 2 : 3) tvc_cols_phased_
   for (int r = t; r < w * VEC; r += kPhT) {
     const int64_t qr = (int64_t)blockIdx.x * w + r / VEC;
     if (qr >= a.u * pps) break;
-    const int64_t ir = (qr >> 32) ? qr / pps : (int64_t)((uint32_t)qr / (uint32_t)pps);
+    const int64_t ir = piece_row(qr, pps);
     const int64_t lr = (qr - ir * pps) * VEC + r % VEC;
     if (lr >= a.v) continue;
     if constexpr (kF64Acc<DT>) {

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(kRgThreads, kRgBlocks<DT>) tvc_cols_ragged_ker
   constexpr int ES = E::kSize, VEC = 16 / ES;
   const int64_t q = (int64_t)blockIdx.x * kRgThreads + threadIdx.x;
   if (q >= a.u * pps) return;
-  const int64_t i = (q >> 32) ? q / pps : (int64_t)((uint32_t)q / (uint32_t)pps);
+  const int64_t i = piece_row(q, pps);
   const int64_t l = (q - i * pps) * VEC;
   const int nv = (int)min((int64_t)VEC, a.v - l), bytes = nv * ES;
   const int64_t j0 = (int64_t)blockIdx.y * a.chunk, j1 = min(a.nk, j0 + a.chunk);
