@@ -56,7 +56,8 @@ struct HgArgs {
   void* parts[2];     // partial sums of z_j: blocks + max n each
 };
 
-// Waits until every block has arrived `want` times in all; false when the
+// Waits for `want` arrivals in all (counted modulo 2^32: ten million sweeps of
+// three modes pass it); false when the
 // wait gave up (the error word is set, the block leaves).
 __device__ bool grid_barrier(unsigned* arrived, unsigned want, int* flag) {
   __syncthreads();
@@ -68,7 +69,7 @@ __device__ bool grid_barrier(unsigned* arrived, unsigned want, int* flag) {
     unsigned v;
     for (;;) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrived) : "memory");
-      if (v >= want) break;
+      if (arrivals_reached(v, want)) break;
       if (clock64() - t0 > kHgWaitLimit) {
         atomicExch(&g_hopm_grid_error, kHgError);
         ok = false;

@@ -18,4 +18,8 @@ TVCG_HD int64_t piece_row(int64_t q, int64_t n) {
   return ((q | n) >> 32) ? q / n : (int64_t)((uint32_t)q / (uint32_t)n);
 }
 
+// Whether a count of barrier arrivals `v` has reached `want`, both modulo 2^32
+// and less than 2^31 apart.
+TVCG_HD bool arrivals_reached(uint32_t v, uint32_t want) { return (int32_t)(v - want) >= 0; }
+
 }  // namespace tvcg
