@@ -8,8 +8,8 @@
 // gx, v == 1 and k > 0: gx = (A viewed as u x n_k) x_0 gy, i.e. a TVC of
 //   mode 0 on the unfolded view (the column kernel), with gy times the slab
 //   scale for narrow storage.
-// gx, otherwise: each thread owns a 16-byte piece of columns (i, l), keeps
-//   its gy in registers and streams the piece's rows, eight (rows off 16-byte
+// gx, otherwise: each thread owns 16-byte pieces of columns (i, l), keeps
+//   their gy in registers (FP64 arithmetic: in shared memory) and streams the piece's rows, eight (rows off 16-byte
 //   boundaries: four) in flight; a warp reduces the rows' dot products over
 //   its lanes with halving exchanges into its own sums of a chunk of rows in
 //   shared memory.  Blocks walk the pieces persistently and leave one partial
@@ -40,7 +40,7 @@ struct GradArgs {
   void* partial;    // [nblk][nk], vector type
   int64_t u, nk, v, upi0, pps, nblk;
   int mode0;
-  int rch;          // rows per chunk (<= kGxRows)
+  int rch;          // rows per chunk (<= kGxRows, kGx64Rows)
 };
 
 // ------------------------------------------------------------- gx, v >= 2
@@ -78,36 +78,45 @@ __device__ __forceinline__ float gx_lanes(float (&a)[M]) {
   return r;
 }
 
-// The same for float-float pairs (TwoSum per exchange).
+// The same for float-float pairs (s, c), joined into (s, c, e): with the error
+// of c kept too, since c alone loses 2^-48 of the sum at every exchange.
 template <int M>
-__device__ __forceinline__ void gx_lanes(float (&s)[M], float (&c)[M]) {
+__device__ __forceinline__ void gx_lanes(float (&s)[M], float (&c)[M], float& e0) {
   const int lane = threadIdx.x & 31;
-  auto join = [](float& s0, float& c0, float s1, float c1) {
-    float t, err;
-    two_sum(s0, s1, t, err);
+  float e[M];
+#pragma unroll
+  for (int q = 0; q < M; q++) e[q] = 0.0f;
+  auto join = [](float& s0, float& c0, float& r0, float s1, float c1, float r1) {
+    float t, es, ec, et;
+    two_sum(s0, s1, t, es);
     s0 = t;
-    c0 = __fadd_rn(__fadd_rn(c0, c1), err);
+    two_sum(c0, c1, t, ec);
+    two_sum(t, es, c0, et);
+    r0 = __fadd_rn(__fadd_rn(r0, r1), __fadd_rn(ec, et));
   };
 #pragma unroll
   for (int h = M / 2, bit = 16; h >= 1; h >>= 1, bit >>= 1) {
     const bool up = lane & bit;
 #pragma unroll
-    for (int e = 0; e < h; e++) {
-      const float os = up ? s[e] : s[e + h], oc = up ? c[e] : c[e + h];
-      s[e] = up ? s[e + h] : s[e];
-      c[e] = up ? c[e + h] : c[e];
-      join(s[e], c[e], __shfl_xor_sync(0xFFFFFFFFu, os, bit), __shfl_xor_sync(0xFFFFFFFFu, oc, bit));
+    for (int q = 0; q < h; q++) {
+      const float os = up ? s[q] : s[q + h], oc = up ? c[q] : c[q + h], oe = up ? e[q] : e[q + h];
+      s[q] = up ? s[q + h] : s[q];
+      c[q] = up ? c[q + h] : c[q];
+      e[q] = up ? e[q + h] : e[q];
+      join(s[q], c[q], e[q], __shfl_xor_sync(0xFFFFFFFFu, os, bit), __shfl_xor_sync(0xFFFFFFFFu, oc, bit),
+           bit == 16 ? 0.0f : __shfl_xor_sync(0xFFFFFFFFu, oe, bit));
     }
   }
 #pragma unroll
   for (int bit = 16 / M; bit >= 1; bit >>= 1)
-    join(s[0], c[0], __shfl_xor_sync(0xFFFFFFFFu, s[0], bit), __shfl_xor_sync(0xFFFFFFFFu, c[0], bit));
+    join(s[0], c[0], e[0], __shfl_xor_sync(0xFFFFFFFFu, s[0], bit), __shfl_xor_sync(0xFFFFFFFFu, c[0], bit),
+         __shfl_xor_sync(0xFFFFFFFFu, e[0], bit));
+  e0 = e[0];
 }
 
 // Bound: HBM.  128^4 FP32, modes 0-2: 190 us and a reduction of 15 -> 163 and
 // 3 (7.0 TB/s; the kernel before held 16 rows' sums and loads in 168
-// registers, one block per SM); 17x52x68x18x31 FP64 mode 1 127 -> 79 us,
-// 12x93x44x11x82 FP32 mode 3 136 -> 62.  Resident blocks per SM (the grid is
+// registers, one block per SM); 12x93x44x11x82 FP32 mode 3 136 -> 62 us.  Resident blocks per SM (the grid is
 // one wave of them):
 template <tvc_dtype DT>
 inline constexpr int kGxBlocks = DT == TVC_E4M3 ? 2 : 3;
@@ -116,17 +125,13 @@ inline constexpr int kGxBlocks = DT == TVC_E4M3 ? 2 : 3;
 template <tvc_dtype DT, bool AL>
 __global__ void __launch_bounds__(kBT, kGxBlocks<DT>) tvc_gradx_kernel(const GradArgs<DT> a) {
   using E = Elem<DT>;
-  using T = typename E::T;
-  using V = typename E::V;
-  constexpr bool F64 = kF64Acc<DT>;
   constexpr int ES = E::kSize, VEC = 16 / ES, RB = AL ? 8 : 4;
-  using Sum = std::conditional_t<F64, double, float2>;  // float2: compensated pair
-  __shared__ Sum sums[kBW][kGxRows];
+  __shared__ float2 sums[kBW][kGxRows];  // compensated pairs
   const int64_t b = blockIdx.x % a.nblk, j0 = blockIdx.x / a.nblk * a.rch;
   const int jn = (int)min((int64_t)a.rch, a.nk - j0);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  Sum* const mine = sums[warp];
-  for (int j = lane; j < jn; j += 32) mine[j] = Sum{};
+  float2* const mine = sums[warp];
+  for (int j = lane; j < jn; j += 32) mine[j] = make_float2(0.0f, 0.0f);
   __syncwarp();
   const uint64_t sb = (uint64_t)a.v * ES;
   const int64_t pieces = a.u * a.pps;
@@ -136,23 +141,14 @@ __global__ void __launch_bounds__(kBT, kGxBlocks<DT>) tvc_gradx_kernel(const Gra
     const int64_t i = ok ? piece_row(q, a.pps) : 0;
     const int64_t l = ok ? (q - i * a.pps) * VEC : 0;
     const int nv = ok ? (int)min((int64_t)VEC, a.v - l) : 0, bytes = nv * ES;
-    const uint64_t ad0 = reinterpret_cast<uint64_t>(a.A) + (uint64_t)((i * a.nk + j0) * a.v + l) * ES;
-    const V* const gyp = static_cast<const V*>(a.gy) + i * a.v + l;
-    // gy of the piece (zero past the row): split pieces, or FP32 with the slab scale
-    XSplit gs[F64 ? VEC : 1];
-    float gf[F64 ? 1 : VEC];
-    if constexpr (F64) {
-#pragma unroll
-      for (int e = 0; e < VEC; e++) gs[e] = e < nv ? split_x(__ldg(gyp + e)) : XSplit{0.0f, 0.0f};
-    } else {
-      float sc = 1.0f;
-      if constexpr (kNarrow<DT>) {
-        if (!a.mode0 && a.scales) sc = __ldg(a.scales + i / a.upi0);
-      }
-#pragma unroll
-      for (int e = 0; e < VEC; e++) gf[e] = e < nv ? __fmul_rn(__ldg(gyp + e), sc) : 0.0f;
+    uint64_t ad = reinterpret_cast<uint64_t>(a.A) + (uint64_t)((i * a.nk + j0) * a.v + l) * ES;
+    const float* const gyp = static_cast<const float*>(a.gy) + i * a.v + l;
+    float gf[VEC], sc = 1.0f;  // gy of the piece times the slab scale (zero past the row)
+    if constexpr (kNarrow<DT>) {
+      if (!a.mode0 && a.scales) sc = __ldg(a.scales + i / a.upi0);
     }
-    uint64_t ad = ad0;
+#pragma unroll
+    for (int e = 0; e < VEC; e++) gf[e] = e < nv ? __fmul_rn(__ldg(gyp + e), sc) : 0.0f;
     for (int j = 0; j < jn; j += RB) {
       Chunks ch[RB];
       uint32_t sh[RB];
@@ -168,85 +164,293 @@ __global__ void __launch_bounds__(kBT, kGxBlocks<DT>) tvc_gradx_kernel(const Gra
         sh[e] = (uint32_t)ad & 15;
         ad += sb;
       }
-      if constexpr (F64) {
-        float s[RB], c[RB];
-        uint32_t bad = 0;
+      float s[RB];
 #pragma unroll
-        for (int e = 0; e < RB; e++) {
-          typename E::C r[VEC];
-          gx_piece<DT>(AL ? ch[e].a : cut<ES>(ch[e], sh[e]), r);
-          s[e] = c[e] = 0.0f;
-          if (j + e < jn) {
+      for (int e = 0; e < RB; e++) {
+        float r[VEC];
+        gx_piece<DT>(AL ? ch[e].a : cut<ES>(ch[e], sh[e]), r);
+        if (nv < VEC) {  // what follows the row is another row
 #pragma unroll
-            for (int x = 0; x < VEC; x++)
-              if (x < nv) df_step(s[e], c[e], bad, r[x], gs[x]);
-          }
-          bad |= isfinite(__fadd_rn(s[e], c[e])) ? 0u : 1u;
+          for (int x = 0; x < VEC; x++) r[x] = x < nv ? r[x] : 0.0f;
         }
-        if (__any_sync(0xFFFFFFFFu, bad != 0)) {
-          // an element or an entry of gy outside the exact window: these
-          // rows again with FP64 multiply-adds
-          for (int e = 0; e < RB && j + e < jn; e++) {
-            double d = 0.0;
-            for (int x = 0; x < nv; x++)
-              d = fma((double)*reinterpret_cast<const T*>(ad0 + (uint64_t)(j + e) * sb + x * ES), __ldg(gyp + x), d);
+        s[e] = 0.0f;
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, off);
-            if (lane == 0) mine[j + e] += d;
-          }
-          __syncwarp();
-        } else {
-          gx_lanes<RB>(s, c);
-          const int row = lane / (32 / RB);
-          if (lane % (32 / RB) == 0 && j + row < jn) mine[j + row] += (double)s[0] + (double)c[0];
-          __syncwarp();
-        }
-      } else {
-        float s[RB];
-#pragma unroll
-        for (int e = 0; e < RB; e++) {
-          float r[VEC];
-          gx_piece<DT>(AL ? ch[e].a : cut<ES>(ch[e], sh[e]), r);
-          if (nv < VEC) {  // what follows the row is another row
-#pragma unroll
-            for (int x = 0; x < VEC; x++) r[x] = x < nv ? r[x] : 0.0f;
-          }
-          s[e] = 0.0f;
-#pragma unroll
-          for (int x = 0; x < VEC; x++) s[e] = __fmaf_rn(r[x], gf[x], s[e]);
-        }
-        const float v = gx_lanes<RB>(s);
-        const int row = lane / (32 / RB);
-        if (lane % (32 / RB) == 0 && j + row < jn) {
-          const float2 o = mine[j + row];
-          float sum, err;
-          two_sum(o.x, v, sum, err);
-          mine[j + row] = make_float2(sum, __fadd_rn(o.y, err));
-        }
-        __syncwarp();
+        for (int x = 0; x < VEC; x++) s[e] = __fmaf_rn(r[x], gf[x], s[e]);
       }
+      const float v = gx_lanes<RB>(s);
+      const int row = lane / (32 / RB);
+      if (lane % (32 / RB) == 0 && j + row < jn) {
+        const float2 o = mine[j + row];
+        float sum, err;
+        two_sum(o.x, v, sum, err);
+        mine[j + row] = make_float2(sum, __fadd_rn(o.y, err));
+      }
+      __syncwarp();
     }
   }
   __syncthreads();
   for (int j = t; j < jn; j += kBT) {
-    V val;
-    if constexpr (F64) {
-      val = sums[0][j];
-      for (int w = 1; w < kBW; w++) val += sums[w][j];
-    } else {
-      KahanF32 k;
-      for (int w = 0; w < kBW; w++) {
-        const float2 o = sums[w][j];
-        k.add(o.x);
-        k.add(o.y == o.y ? o.y : 0.0f);  // NaN: o.x alone (see pair_value)
-      }
-      val = k.value();
-      if constexpr (kNarrow<DT>) {
-        if (a.mode0 && a.scales) val = __fmul_rn(val, __ldg(a.scales + j0 + j));
+    KahanF32 k;
+    for (int w = 0; w < kBW; w++) {
+      const float2 o = sums[w][j];
+      k.add(o.x);
+      k.add(o.y == o.y ? o.y : 0.0f);  // NaN: o.x alone (see pair_value)
+    }
+    float val = k.value();
+    if constexpr (kNarrow<DT>) {
+      if (a.mode0 && a.scales) val = __fmul_rn(val, __ldg(a.scales + j0 + j));
+    }
+    static_cast<float*>(a.partial)[b * a.nk + j0 + j] = val;
+  }
+}
+
+// The same in FP64.
+template <int M>
+__device__ __forceinline__ double gx_lanes(double (&a)[M]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = M / 2, bit = 16; h >= 1; h >>= 1, bit >>= 1) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int e = 0; e < h; e++) {
+      const double mine = up ? a[e + h] : a[e], other = up ? a[e] : a[e + h];
+      a[e] = mine + __shfl_xor_sync(0xFFFFFFFFu, other, bit);
+    }
+  }
+  double r = a[0];
+#pragma unroll
+  for (int bit = 16 / M; bit >= 1; bit >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, bit);
+  return r;
+}
+
+// FP64 arithmetic (FP64 and single-double storage): a thread adds the
+// float-float products of a row over the kp pieces of its tile (256 kp pieces)
+// before they are joined over the lanes, so that the exchanges and the FP64
+// sums behind them are paid once per kp pieces.
+// An element outside the exact window enters the pairs as zero and an FP64
+// sum of the thread (its slots) by a multiply-add; exact zeros need neither.  gy
+// outside its window (a mean loss over a large tensor is) is first scaled by a
+// power of two per warp and tile.
+// Bound: latency and the FP32 pipe.  us of gx on 17x52x68x18x31 mode 1 / 128x128x128x16
+// mode 1 / 300x200x256 mode 0 / 40x21x33000 mode 1, FP64: 93 / 87 / 47 / 84
+// (2.9-3.4 TB/s); 1% zeros the same; 1% of the elements nonzero and below 2^-64
+// 157 / 149 / 80 / 139; all of them 204 / 191 / 101 / 174; gy below 2^-32 93 / 87
+// / 47 / 84.  Single-double: 75 / 68 / 43 / 66.  A kernel that joined the lanes
+// in plain pairs after every piece took 80 / 84 / 44 / 73 on plain data, 336 /
+// 386 / 175 / 284 with 1% zeros or a small gy, and was up to nine times further
+// off (480x161 mode 0: 1.6e-14 of the terms' root sum of squares, 2.8e-15 here).
+template <tvc_dtype DT>
+inline constexpr int kGxTile = DT == TVC_F64 ? 4 : 2;  // pieces per thread and tile at most (48 KB of shared memory)
+constexpr int kGx64Rows = 128;                          // rows per chunk at most
+constexpr int kGx64Blocks = 3;                          // resident per SM (2: up to 7% slower, 4: 15-30%)
+
+// ah + al of an element, both zero outside the window; `out` collects the bits
+// of nonzero elements there.
+__device__ __forceinline__ void gx_split(double v, float& ah, float& al, uint32_t& out) {
+  const uint32_t lo = (uint32_t)__double2loint(v), hi = (uint32_t)__double2hiint(v);
+  const bool in = hi * 2u - kDfWindowBase < (1u << 28);
+  const uint32_t hb = in ? __funnelshift_l(lo, hi - 0x38000000u, 3) | (hi & 0x80000000u) : 0u;
+  ah = __uint_as_float(hb);
+  al = __fmul_rn(__uint2float_rn(in ? lo & 0x1FFFFFFFu : 0u), __uint_as_float((hb & 0xFF800000u) - 0x1A000000u));
+  if (!in) out |= hi * 2u | lo;
+}
+__device__ __forceinline__ void gx_split(float v, float& ah, float& al, uint32_t& out) {
+  const bool in = df_out_of_window(v) == 0;
+  ah = in ? v : 0.0f;
+  al = 0.0f;
+  if (!in) out |= __float_as_uint(v) << 1;
+}
+
+// split_x of an entry in the window, or zero, by integer operations (its
+// conversions and subtraction in FP64 cost a tenth of the kernel): the entry
+// rounded to 24 bits, and the signed rest.
+__device__ __forceinline__ XSplit gx_split_gy(double g) {
+  const uint64_t w = (uint64_t)__double_as_longlong(g);
+  if (w << 1 == 0) return XSplit{0.0f, 0.0f};
+  const uint64_t r = w + (1u << 28);
+  const uint32_t lo = (uint32_t)r, hi = (uint32_t)(r >> 32);
+  XSplit p;
+  p.xh = __uint_as_float(__funnelshift_l(lo, hi - 0x38000000u, 3) | (hi & 0x80000000u));
+  // units of 2^-52 of the unrounded exponent
+  const uint32_t unit = (((uint32_t)(w >> 32) - 0x38000000u) << 3 & 0x7F800000u) - 0x1A000000u;
+  const float rest = __int2float_rn((int)(lo & 0x1FFFFFFFu) - (1 << 28));
+  p.xl = __fmul_rn((int64_t)w < 0 ? -rest : rest, __uint_as_float(unit));
+  return p;
+}
+
+__device__ __forceinline__ double gx_dfma(double a, const double* g, double d) { return dfma_slow(a, g, d); }
+__device__ __forceinline__ double gx_dfma(float a, const double* g, double d) { return dfma_slow_f(a, g, d); }
+
+template <tvc_dtype DT, bool AL>
+__global__ void __launch_bounds__(kBT, kGx64Blocks) tvc_gradx64_kernel(const GradArgs<DT> a) {
+  using E = Elem<DT>;
+  using T = typename E::T;
+  constexpr int ES = E::kSize, VEC = 16 / ES, RB = AL ? 8 : 4, KP = kGxTile<DT>;
+  extern __shared__ __align__(16) unsigned char gx_smem[];
+  double* const sums = reinterpret_cast<double*>(gx_smem);            // [kBW][kGx64Rows]
+  double* const slots = sums + kBW * kGx64Rows;                       // [RB][kBT]
+  int64_t* const offs = reinterpret_cast<int64_t*>(slots + RB * kBT);  // [KP][kBT]: 8 * element of row 0 + elements inside the row, < 0: no piece
+  float2* const gsm = reinterpret_cast<float2*>(offs + KP * kBT);     // [KP][VEC][kBT]: split gy
+  const int64_t b = blockIdx.x % a.nblk, j0 = blockIdx.x / a.nblk * a.rch;
+  const int jn = (int)min((int64_t)a.rch, a.nk - j0);
+  const int t = threadIdx.x, lane = t & 31;
+  double* const mine = sums + (t >> 5) * kGx64Rows;
+  double* const slot = slots + t;
+  for (int j = lane; j < jn; j += 32) mine[j] = 0.0;
+#pragma unroll
+  for (int e = 0; e < RB; e++) slot[e * kBT] = 0.0;
+  __syncwarp();
+  const T* const A = static_cast<const T*>(a.A) + j0 * a.v;
+  const double* const gy = static_cast<const double*>(a.gy);
+  // an even share of the pieces per block
+  const int64_t pieces = a.u * a.pps, qe = pieces * (b + 1) / a.nblk;
+  for (int64_t q0 = pieces * b / a.nblk; q0 < qe; q0 += KP * kBT) {
+    const int kp = (int)min((int64_t)KP, (qe - q0 + kBT - 1) / kBT);
+    // the thread's pieces and their gy
+    uint32_t gout = 0;   // VEC bits per piece: entries that stay outside the window
+    double scale = 1.0;  // of the warp's pairs
+    double g[KP][VEC];
+    int most = 0;        // exponent field of the largest entry below 2^1000
+    bool in = true;
+    auto inside = [](double v) {  // the window of an entry, or zero
+      const uint32_t hi = (uint32_t)__double2hiint(v) << 1, lo = (uint32_t)__double2loint(v);
+      return hi - ((1023u - 32) << 21) < (64u << 21) || (hi | lo) == 0;
+    };
+#pragma unroll
+    for (int k = 0; k < KP; k++) {
+      const int64_t q = q0 + k * kBT + t;
+      const bool ok = q < qe;
+      const int64_t i = ok ? piece_row(q, a.pps) : 0, l = ok ? (q - i * a.pps) * VEC : 0;
+      offs[k * kBT + t] = ok ? (i * a.nk * a.v + l) * 8 + min((int64_t)VEC, a.v - l) : -1;
+#pragma unroll
+      for (int x = 0; x < VEC; x++) {
+        g[k][x] = ok && l + x < a.v ? __ldg(gy + i * a.v + l + x) : 0.0;
+        const int f = __double2hiint(g[k][x]) >> 20 & 0x7FF;
+        if (f < 2023) most = max(most, f);
+        in = in && inside(g[k][x]);
       }
     }
-    static_cast<V*>(a.partial)[b * a.nk + j0 + j] = val;
+    if (!__all_sync(0xFFFFFFFFu, in)) {
+      most = __reduce_max_sync(0xFFFFFFFFu, most);
+      if (most > 23) {
+        // the power of two that takes the largest entry to [1, 2), and back
+        scale = __hiloint2double(most << 20, 0);
+        const double down = __hiloint2double((2046 - most) << 20, 0);
+#pragma unroll
+        for (int k = 0; k < KP; k++)
+#pragma unroll
+          for (int x = 0; x < VEC; x++) g[k][x] *= down;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < KP; k++)
+#pragma unroll
+      for (int x = 0; x < VEC; x++) {
+        XSplit p{0.0f, 0.0f};
+        if (inside(g[k][x]))
+          p = gx_split_gy(g[k][x]);
+        else
+          gout |= 1u << (k * VEC + x);
+        gsm[(k * VEC + x) * kBT + t] = make_float2(p.xh, p.xl);
+      }
+    for (int j = 0; j < jn; j += RB) {
+      const int rows = min(RB, jn - j);
+      float s[RB], c[RB];
+#pragma unroll
+      for (int e = 0; e < RB; e++) s[e] = c[e] = 0.0f;
+      bool extra = false;
+      for (int k = 0; k < kp; k++) {
+        if (offs[k * kBT + t] < 0) break;
+        const int64_t off = offs[k * kBT + t] >> 3;
+        const int nv = AL ? VEC : (int)(offs[k * kBT + t] & 7);
+        const T* const p = A + off + j * a.v;
+        const uint64_t ad = reinterpret_cast<uint64_t>(p);
+        Chunks ch[RB];
+#pragma unroll
+        for (int e = 0; e < RB; e++) {
+          if constexpr (AL)
+            ch[e].a = e < rows ? __ldcs(reinterpret_cast<const uint4*>(p + e * a.v)) : make_uint4(0u, 0u, 0u, 0u);
+          else {
+            ch[e].a = ch[e].b = make_uint4(0u, 0u, 0u, 0u);
+            if (e < rows) ld_chunks(ad + (uint64_t)(e * a.v) * ES, nv * ES, ch[e]);
+          }
+        }
+        auto row = [&](int e, typename E::C (&r)[VEC]) {
+          gx_piece<DT>(AL ? ch[e].a : cut<ES>(ch[e], (uint32_t)(ad + (uint64_t)(e * a.v) * ES) & 15), r);
+        };
+        XSplit xs[VEC];
+#pragma unroll
+        for (int x = 0; x < VEC; x++) {
+          const float2 w = gsm[(k * VEC + x) * kBT + t];
+          xs[x] = XSplit{w.x, w.y};
+        }
+        uint32_t out = 0;
+#pragma unroll
+        for (int e = 0; e < RB; e++) {
+          typename E::C r[VEC];
+          row(e, r);
+#pragma unroll
+          for (int x = 0; x < VEC; x++) {
+            if (!AL && x >= nv) continue;  // another row's
+            float ah, al;
+            gx_split(r[x], ah, al, out);
+            const float pr = __fmul_rn(ah, xs[x].xh);
+            float er = __fmaf_rn(ah, xs[x].xh, -pr);
+            er = __fmaf_rn(ah, xs[x].xl, er);
+            er = __fmaf_rn(al, xs[x].xh, er);
+            float sum, err;
+            two_sum(s[e], pr, sum, err);
+            s[e] = sum;
+            c[e] = __fadd_rn(c[e], __fadd_rn(err, er));
+          }
+        }
+        const uint32_t go = gout >> (k * VEC) & ((1u << VEC) - 1);
+        if (out | go) {  // what the pairs left out
+          const int64_t q = q0 + k * kBT + t, i = piece_row(q, a.pps);
+          const double* const gp = gy + i * a.v + (q - i * a.pps) * VEC;
+#pragma unroll
+          for (int e = 0; e < RB; e++) {
+            if (e >= rows) break;
+            typename E::C r[VEC];
+            row(e, r);
+#pragma unroll
+            for (int x = 0; x < VEC; x++)
+              if (x < nv && ((go >> x & 1) || (df_out_of_window(r[x]) != 0 && r[x] != 0)))
+                slot[e * kBT] = gx_dfma(r[x], gp + x, slot[e * kBT]);
+          }
+          extra = true;
+        }
+      }
+      float e0;
+      gx_lanes<RB>(s, c, e0);
+      const int row = lane / (32 / RB);
+      double d = ((double)s[0] + (double)c[0]) + (double)e0;
+      if (scale != 1.0) d *= scale;
+      if (__any_sync(0xFFFFFFFFu, extra)) {
+        double w[RB];
+#pragma unroll
+        for (int e = 0; e < RB; e++) {
+          w[e] = slot[e * kBT];
+          slot[e * kBT] = 0.0;
+        }
+        d += gx_lanes<RB>(w);
+      }
+      if (lane % (32 / RB) == 0 && row < rows) mine[j + row] += d;
+      __syncwarp();
+    }
   }
+  __syncthreads();
+  for (int j = t; j < jn; j += kBT) {
+    double val = sums[j];
+    for (int w = 1; w < kBW; w++) val += sums[w * kGx64Rows + j];
+    static_cast<double*>(a.partial)[b * a.nk + j0 + j] = val;
+  }
+}
+
+// Shared memory of that kernel.
+template <tvc_dtype DT, bool AL>
+constexpr int gx64_smem() {
+  return (kBW * kGx64Rows + (AL ? 8 : 4) * kBT) * 8 + kGxTile<DT> * kBT * (8 + 16 / Elem<DT>::kSize * 8);
 }
 
 // gx[j] = the blocks' partial sums in FP64, 32 entries per block: each warp a
@@ -390,11 +594,34 @@ GxPlan plan_gx(const Shape& s, tvc_dtype dt, const void* A) {
   // One wave of blocks: chunks of 256 rows, or fewer (down to 32) where the
   // pieces alone do not fill it.
   const int64_t wave = (int64_t)device_sms() * (dt == TVC_E4M3 ? kGxBlocks<TVC_E4M3> : kGxBlocks<TVC_F32>);
-  const int64_t tiles = cdiv(s.u * g.pps, kBT);
-  g.nchunks = std::max(cdiv(s.nk, kGxRows), std::min(cdiv(s.nk, 32), wave / tiles));
-  g.rch = (int)(cdiv(cdiv(s.nk, g.nchunks), 8) * 8);
-  g.nchunks = cdiv(s.nk, g.rch);
-  g.nblk = std::max<int64_t>(1, std::min(tiles, wave / g.nchunks));
+  const int64_t pieces = s.u * g.pps, tiles = cdiv(pieces, kBT);
+  if (vs == 8) {
+    const int64_t wave = (int64_t)device_sms() * kGx64Blocks;
+    // FP64 arithmetic: the cut of the rows that leaves the shortest block, in
+    // rows of 256 pieces (the preparation of gy costs about two)
+    int64_t cost = INT64_MAX;
+    for (int64_t n = cdiv(s.nk, kGx64Rows); n <= std::min(wave, std::max(cdiv(s.nk, kGx64Rows), cdiv(s.nk, 16))); n++) {
+      const int64_t rch = cdiv(cdiv(s.nk, n), 8) * 8, nch = cdiv(s.nk, rch);
+      const int64_t nblk = std::max<int64_t>(1, std::min(tiles, wave / nch));
+      const int64_t c = cdiv(cdiv(pieces, nblk), kBT) * (rch + 2) * std::max<int64_t>(1, cdiv(nch * nblk, wave));
+      if (c < cost) {
+        cost = c;
+        g.rch = (int)rch;
+        g.nchunks = nch;
+        g.nblk = nblk;
+      }
+    }
+    if (cost == INT64_MAX) {  // more chunks than a wave
+      g.rch = kGx64Rows;
+      g.nchunks = cdiv(s.nk, g.rch);
+      g.nblk = 1;
+    }
+  } else {
+    g.nchunks = std::max(cdiv(s.nk, kGxRows), std::min(cdiv(s.nk, 32), wave / tiles));
+    g.rch = (int)(cdiv(cdiv(s.nk, g.nchunks), 8) * 8);
+    g.nchunks = cdiv(s.nk, g.rch);
+    g.nblk = std::max<int64_t>(1, std::min(tiles, wave / g.nchunks));
+  }
   g.ws_partial = align_up((size_t)g.nblk * s.nk * vs, 256);
   g.total = g.ws_partial;
   return g;
@@ -418,10 +645,17 @@ tvc_status run_gx(const GxPlan& g, const Shape& s, const void* A, const void* gy
   a.mode0 = s.mode == 0;
   a.rch = g.rch;
   const unsigned grid = (unsigned)(g.nblk * g.nchunks);
-  if (g.al)
-    tvc_gradx_kernel<DT, true><<<grid, kBT, 0, st>>>(a);
-  else
-    tvc_gradx_kernel<DT, false><<<grid, kBT, 0, st>>>(a);
+  if constexpr (kF64Acc<DT>) {
+    if (g.al)
+      tvc_gradx64_kernel<DT, true><<<grid, kBT, gx64_smem<DT, true>(), st>>>(a);
+    else
+      tvc_gradx64_kernel<DT, false><<<grid, kBT, gx64_smem<DT, false>(), st>>>(a);
+  } else {
+    if (g.al)
+      tvc_gradx_kernel<DT, true><<<grid, kBT, 0, st>>>(a);
+    else
+      tvc_gradx_kernel<DT, false><<<grid, kBT, 0, st>>>(a);
+  }
   tvc_gradx_reduce_kernel<V><<<(unsigned)cdiv(s.nk, 32), kBT, 0, st>>>(static_cast<const V*>(ws), static_cast<V*>(gx), s.nk, g.nblk);
   count_launches(2);
   return cuda_status(cudaGetLastError());

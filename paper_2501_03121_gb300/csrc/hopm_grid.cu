@@ -56,9 +56,9 @@ struct HgArgs {
   void* parts[2];     // partial sums of z_j: blocks + max n each
 };
 
-// Waits for `want` arrivals in all (counted modulo 2^32: ten million sweeps of
-// three modes pass it); false when the
-// wait gave up (the error word is set, the block leaves).
+// Waits for `want` arrivals in all, counted modulo 2^32 (ten million sweeps of
+// three modes pass it); false when the wait gave up (the error word is set, the
+// block leaves).
 __device__ bool grid_barrier(unsigned* arrived, unsigned want, int* flag) {
   __syncthreads();
   if (threadIdx.x == 0) {
