@@ -227,7 +227,24 @@ constexpr int64_t kGxJ = 256;        // rows j per warp-mapped item
 constexpr int kFusedRows = 512;      // rows n_k up to which columns are fused
 constexpr int kFusedRowMax = 256;    // row lengths of the fused rows (v == 1)
 constexpr int kFusedRowMin = 32;
+// A warp's row sums of a fused item are compensated pairs, the errors kErr
+// behind the sums.  More than kErr rows need none: the item is then at most
+// 1024 columns (fused_per), one sum per warp and row.
+constexpr int kErr = kFusedRows / 2;
+static_assert(kFusedRowMax <= kErr && (1 << 19) / (kErr + 1) < 2 * 1024, "one sum per row above kErr rows");
 
+// A term into a compensated pair (p[0], p[kErr]), and a pair (or its sum alone)
+// into a compensated sum.
+__device__ __forceinline__ void add_pair(float* p, float v) {
+  float t, err;
+  two_sum(p[0], v, t, err);
+  p[0] = t;
+  p[kErr] = __fadd_rn(p[kErr], err);
+}
+__device__ __forceinline__ void add_pair(KahanF32& s, const float* p, bool pair) {
+  s.add(p[0]);
+  if (pair) s.add(p[kErr] == p[kErr] ? p[kErr] : 0.0f);  // NaN: p[0] alone (see pair_value)
+}
 
 // After an item's partial sums of gx are written: the tensor's last item
 // adds the gxk partials in order and resets the counter.
@@ -426,9 +443,9 @@ __device__ __forceinline__ void st_vec(float* p, const float (&v)[VEC], float m)
 // into its own row of red; gA = gy x_j is written on the way.  Bound: one read
 // of A and one write of gA (three passes over memory with an item kind per
 // result).  512 tensors (2.1e9 elements) with all three results, with
-// blk_rows_fused and the smaller items: 7.89 -> 4.46 ms; 40 tensors 3.5 ->
-// 0.42 ms.
-template <int VEC>
+// blk_rows_fused and the smaller items: 7.89 -> 4.52 ms; 40 tensors 3.5 ->
+// 0.43 ms (plain row sums 4.46 and 0.43).
+template <int VEC, bool ONE>
 __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, int items, int* cnt, float* partials,
                                float* red, float* xsm, int* flag) {
   constexpr int RB = VEC == 1 ? 16 : 8, NQ = 4 / VEC;
@@ -437,11 +454,12 @@ __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, 
   const int64_t v = it.v;
   const bool wy = it.y != nullptr, wgx = it.gx != nullptr, wgA = it.gA != nullptr;
   const bool small = it.u * v <= 0xFFFFFFFFll;  // 32-bit division of the columns
-  float* const rw = red + wid * kFusedRows;
+  float* const rw = red + wid * kFusedRows;  // the warp's row sums (pairs, see kErr)
+  const bool pairs = nk <= kErr;
   if (wy || wgA)
     for (int j = t; j < nk; j += kBBT) xsm[j] = __ldg(it.x + j);
   if (wgx)
-    for (int j = lane; j < nk; j += 32) rw[j] = 0.0f;
+    for (int j = lane; j < (pairs ? kErr + nk : nk); j += 32) rw[j] = 0.0f;
   __syncthreads();
   const int nbat = (nk + RB - 1) / RB, per = (nk + nbat - 1) / nbat;
   for (int64_t g = c0 + wid * 128; g < c1; g += (kBBT / 32) * 128) {
@@ -484,7 +502,8 @@ __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, 
 #pragma unroll
               for (int c = 0; c < VEC; c++) {
                 if (e < nb) y0[q][c] = __fmaf_rn(a[e][c], xa, y0[q][c]);
-                if (e + 1 < nb) y1[q][c] = __fmaf_rn(a[e + 1][c], xb, y1[q][c]);
+                float& odd = ONE ? y0[q][c] : y1[q][c];
+                if (e + 1 < nb) odd = __fmaf_rn(a[e + 1][c], xb, odd);
               }
             }
           }
@@ -504,7 +523,12 @@ __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, 
       if (wgx) {
         const float sum = warp_add_many<RB>(acc);
         const int row = lane / (32 / RB);
-        if (lane % (32 / RB) == 0 && row < nb) rw[jb + row] += sum;
+        if (lane % (32 / RB) == 0 && row < nb) {
+          if (pairs)
+            add_pair(rw + jb + row, sum);
+          else
+            rw[jb + row] = sum;
+        }
         __syncwarp();
       }
     }
@@ -523,7 +547,7 @@ __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, 
     for (int j = t; j < nk; j += kBBT) {
       KahanF32 sum;
 #pragma unroll
-      for (int w = 0; w < kBBT / 32; w++) sum.add(red[w * kFusedRows + j]);
+      for (int w = 0; w < kBBT / 32; w++) add_pair(sum, red + w * kFusedRows + j, pairs);
       dst[j] = sum.value();
     }
     finish_gx(it, items, cnt, partials, flag);
@@ -546,6 +570,17 @@ __device__ void blk_rows_fused(const BItem& it, int64_t i0, int64_t i1, int ks, 
     xq[q] = ((wy || wgA) && q * 32 + lane < nk) ? __ldg(it.x + q * 32 + lane) : 0.0f;
     cs[q] = 0.0f;
   }
+  float* const cw = red + wid * kFusedRows + lane;  // the lane's column sums (pairs), folded every 64 rows
+#pragma unroll
+  for (int q = 0; q < NC; q++) cw[q * 32] = cw[q * 32 + kErr] = 0.0f;
+  auto fold = [&]() {
+#pragma unroll
+    for (int q = 0; q < NC; q++) {
+      add_pair(cw + q * 32, cs[q]);
+      cs[q] = 0.0f;
+    }
+  };
+  int blk = 0;
   for (int64_t i = i0 + wid * RB; i < i1; i += (kBBT / 32) * RB) {
     const int nb = (int)min((int64_t)RB, i1 - i);
     float pe[RB], acc[RB];
@@ -589,17 +624,19 @@ __device__ void blk_rows_fused(const BItem& it, int64_t i0, int64_t i1, int ks, 
       const int row = lane / (32 / RB);
       if (lane % (32 / RB) == 0 && row < nb) it.y[i + row] = sum;
     }
+    if (wgx && ++blk == 64 / RB) {
+      fold();
+      blk = 0;
+    }
   }
   if (wgx) {
-#pragma unroll
-    for (int q = 0; q < NC; q++)
-      if (q * 32 + lane < nk) red[wid * kFusedRows + q * 32 + lane] = cs[q];
+    fold();
     __syncthreads();
     float* dst = (it.gxk > 1) ? partials + it.gxp + (int64_t)ks * nk : it.gx;
     for (int j = t; j < nk; j += kBBT) {
       KahanF32 sum;
 #pragma unroll
-      for (int w = 0; w < kBBT / 32; w++) sum.add(red[w * kFusedRows + j]);
+      for (int w = 0; w < kBBT / 32; w++) add_pair(sum, red + w * kFusedRows + j, true);
       dst[j] = sum.value();
     }
     finish_gx(it, items, cnt, partials, flag);
@@ -621,12 +658,21 @@ __global__ void __launch_bounds__(kBBT, kBBlocksPerSM) tvc_batched_kernel(const 
       blk_tvc(it.A, it.u, it.nk, it.v, it.x, it.y, it.gf, wi.a0, wi.a1);
     else if (wi.kind == 3) {
       const uintptr_t al = reinterpret_cast<uintptr_t>(it.A) | reinterpret_cast<uintptr_t>(it.gA);
-      if (it.v % 4 == 0 && al % 16 == 0)
-        blk_cols_fused<4>(it, wi.a0, wi.a1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, xsm, &last_flag);
-      else if (it.v % 2 == 0 && al % 8 == 0)
-        blk_cols_fused<2>(it, wi.a0, wi.a1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, xsm, &last_flag);
+      const int vec = it.v % 4 == 0 && al % 16 == 0 ? 4 : it.v % 2 == 0 && al % 8 == 0 ? 2 : 1;
+      int* const cnt = gx_counters + wi.b;
+      if (it.nk < 8) {
+        if (vec == 4)
+          blk_cols_fused<4, true>(it, wi.a0, wi.a1, wi.e0, wi.e1, cnt, gx_partials, red, xsm, &last_flag);
+        else if (vec == 2)
+          blk_cols_fused<2, true>(it, wi.a0, wi.a1, wi.e0, wi.e1, cnt, gx_partials, red, xsm, &last_flag);
+        else
+          blk_cols_fused<1, true>(it, wi.a0, wi.a1, wi.e0, wi.e1, cnt, gx_partials, red, xsm, &last_flag);
+      } else if (vec == 4)
+        blk_cols_fused<4, false>(it, wi.a0, wi.a1, wi.e0, wi.e1, cnt, gx_partials, red, xsm, &last_flag);
+      else if (vec == 2)
+        blk_cols_fused<2, false>(it, wi.a0, wi.a1, wi.e0, wi.e1, cnt, gx_partials, red, xsm, &last_flag);
       else
-        blk_cols_fused<1>(it, wi.a0, wi.a1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, xsm, &last_flag);
+        blk_cols_fused<1, false>(it, wi.a0, wi.a1, wi.e0, wi.e1, cnt, gx_partials, red, xsm, &last_flag);
     } else if (wi.kind == 4)
       blk_rows_fused(it, wi.a0, wi.a1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, &last_flag);
     else if (wi.kind == 1 || wi.kind == 5)
