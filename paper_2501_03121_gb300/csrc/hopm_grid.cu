@@ -310,6 +310,17 @@ __device__ __noinline__ void hg_contract(HgShared<V>& s, const HgPhase& f, const
   }
 }
 
+// A sum in V: compensated in FP32 (z_j of few entries adds hundreds of products
+// per thread, and a part per block), plain in FP64.
+template <class V>
+struct HgSum : KahanF32 {};
+template <>
+struct HgSum<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+
 // The block's products (s.y, or global y times the outer product when they
 // do not fit) summed per entry of z_j into part[z + block].
 template <class V>
@@ -320,8 +331,9 @@ __device__ void hg_parts(HgShared<V>& s, const HgPhase& f, int d, int from, cons
   if (ze - za >= kHgW) {  // short pieces: a warp each
     for (uint32_t z = za + wid; z < ze; z += kHgW) {
       const uint32_t lb = min(f.ob, (z + 1) * R);
-      V a = 0;
-      for (uint32_t o = max(f.oa, z * R) + lane; o < lb; o += 32) a += term(o);
+      HgSum<V> sum;
+      for (uint32_t o = max(f.oa, z * R) + lane; o < lb; o += 32) sum.add(term(o));
+      V a = sum.value();
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, off);
       if (lane == 0) part[z + blockIdx.x] = a;
@@ -330,8 +342,9 @@ __device__ void hg_parts(HgShared<V>& s, const HgPhase& f, int d, int from, cons
   }
   for (uint32_t z = za; z < ze; z++) {
     const uint32_t lb = min(f.ob, (z + 1) * R);
-    V a = 0;
-    for (uint32_t o = max(f.oa, z * R) + t; o < lb; o += kHgT) a += term(o);
+    HgSum<V> sum;
+    for (uint32_t o = max(f.oa, z * R) + t; o < lb; o += kHgT) sum.add(term(o));
+    V a = sum.value();
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, off);
     if (lane == 0) s.wred[z - za][wid] = a;
@@ -447,17 +460,19 @@ __global__ void __launch_bounds__(kHgT, 1) hopm_grid_kernel(const HgArgs a) {
       auto entry = [&](int i) {
         if (last) return __ldcg(part + i);
         const int b0 = s.b0[s.at[j] + i], b1 = s.b1[s.at[j] + i];
-        V z = __ldcg(part + i + b0);
+        HgSum<V> z;
+        z.add(__ldcg(part + i + b0));
         for (int p = b0 + 1; p <= b1; p++)
-          if (f.Q >= (uint32_t)B || hg_first(f.Q, p, B) < hg_first(f.Q, p + 1, B)) z += __ldcg(part + i + p);
-        return z;
+          if (f.Q >= (uint32_t)B || hg_first(f.Q, p, B) < hg_first(f.Q, p + 1, B)) z.add(__ldcg(part + i + p));
+        return z.value();
       };
       const bool many = !last && f.nj <= 64 && f.nj * 4 <= B;  // many parts per entry: a warp each
       if (many) {
         for (int i = t >> 5; i < f.nj; i += kHgW) {
-          V z = 0;
+          HgSum<V> sum;
           for (int p = s.b0[s.at[j] + i] + (t & 31); p <= s.b1[s.at[j] + i]; p += 32)
-            if (hg_first(f.Q, p, B) < hg_first(f.Q, p + 1, B)) z += __ldcg(part + i + p);
+            if (hg_first(f.Q, p, B) < hg_first(f.Q, p + 1, B)) sum.add(__ldcg(part + i + p));
+          V z = sum.value();
 #pragma unroll
           for (int off = 16; off > 0; off >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, off);
           if ((t & 31) == 0) s.zs[i] = z;

@@ -37,3 +37,23 @@ def test_batched_gx_of_rows():
     gx = batch_gx((n, 64), 1, 0, 2.0**25)
     assert abs(gx[0].item() - (2.0**25 + n - 1)) <= 63 + 4 * 2
     assert bool((gx[1:] == n).all())
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2000, 1900), (3, 2, 1200, 1000)])
+def test_power_method_of_few_leading_entries(dims):
+    # z_0[0] = 2^25 + n - 1 and z_0[1] = n: their quotient, to the rounding of
+    # the two entries of x_0, of z_0[0], and of the tree over a block's threads
+    # (nine levels of half a spacing of 2^25, 18 of 3e7, in the first block).
+    n = dims[2] * dims[3]
+    A = torch.ones(dims, device="cuda")
+    A.view(-1)[0] = 2.0**25
+    one = torch.zeros(dims[1], device="cuda")
+    one[0] = 1.0
+    xs = [torch.ones(dims[0], device="cuda"), one] + [torch.ones(m, device="cuda") for m in dims[2:]]
+    ws = torch.empty(tg.hopm_workspace_size(dims, tg.F32), dtype=torch.uint8, device="cuda")
+    before = tg.kernel_launches()
+    r = tg.hopm(A, xs, 1, workspace=ws).check()
+    assert tg.kernel_launches() - before == 1  # the one-launch kernel
+    got = r.x[0][0].double().item() / r.x[0][1].double().item()
+    want = (2.0**25 + n - 1) / n
+    assert abs(got - want) <= 6 * 2.0**-24 * want + 9 * 2 / n
