@@ -246,17 +246,6 @@ __device__ __forceinline__ void add_pair(KahanF32& s, const float* p, bool pair)
   if (pair) s.add(p[kErr] == p[kErr] ? p[kErr] : 0.0f);  // NaN: p[0] alone (see pair_value)
 }
 
-// A term into a compensated pair, and a pair into a compensated sum.
-__device__ __forceinline__ void add_pair(float2& p, float v) {
-  float t, err;
-  two_sum(p.x, v, t, err);
-  p = make_float2(t, __fadd_rn(p.y, err));
-}
-__device__ __forceinline__ void add_pair(KahanF32& s, float2 p) {
-  s.add(p.x);
-  s.add(p.y == p.y ? p.y : 0.0f);  // NaN: p.x alone (see pair_value)
-}
-
 // After an item's partial sums of gx are written: the tensor's last item
 // adds the gxk partials in order and resets the counter.
 __device__ void finish_gx(const BItem& it, int items, int* cnt, const float* partials, int* flag) {
@@ -458,27 +447,19 @@ __device__ __forceinline__ void st_vec(float* p, const float (&v)[VEC], float m)
 // 0.43 ms (plain row sums 4.46 and 0.43).
 template <int VEC, bool ONE>
 __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, int items, int* cnt, float* partials,
-                               float2* red, float* xsm, int* flag) {
+                               float* red, float* xsm, int* flag) {
   constexpr int RB = VEC == 1 ? 16 : 8, NQ = 4 / VEC;
   const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
   const int nk = (int)it.nk;
   const int64_t v = it.v;
   const bool wy = it.y != nullptr, wgx = it.gx != nullptr, wgA = it.gA != nullptr;
   const bool small = it.u * v <= 0xFFFFFFFFll;  // 32-bit division of the columns
-<<<<<<< Updated upstream
   float* const rw = red + wid * kFusedRows;  // the warp's row sums (pairs, see kErr)
   const bool pairs = nk <= kErr;
   if (wy || wgA)
     for (int j = t; j < nk; j += kBBT) xsm[j] = __ldg(it.x + j);
   if (wgx)
     for (int j = lane; j < (pairs ? kErr + nk : nk); j += 32) rw[j] = 0.0f;
-=======
-  float2* const rw = red + wid * kFusedRows;  // compensated sums of the warp's rows
-  if (wy || wgA)
-    for (int j = t; j < nk; j += kBBT) xsm[j] = __ldg(it.x + j);
-  if (wgx)
-    for (int j = lane; j < nk; j += 32) rw[j] = make_float2(0.0f, 0.0f);
->>>>>>> Stashed changes
   __syncthreads();
   const int nbat = (nk + RB - 1) / RB, per = (nk + nbat - 1) / nbat;
   for (int64_t g = c0 + wid * 128; g < c1; g += (kBBT / 32) * 128) {
@@ -521,17 +502,8 @@ __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, 
 #pragma unroll
               for (int c = 0; c < VEC; c++) {
                 if (e < nb) y0[q][c] = __fmaf_rn(a[e][c], xa, y0[q][c]);
-<<<<<<< Updated upstream
                 float& odd = ONE ? y0[q][c] : y1[q][c];
                 if (e + 1 < nb) odd = __fmaf_rn(a[e + 1][c], xb, odd);
-=======
-                if (e + 1 < nb) {  // fewer than eight rows: one chain, a rounding less
-                  if (nk < 8)
-                    y0[q][c] = __fmaf_rn(a[e + 1][c], xb, y0[q][c]);
-                  else
-                    y1[q][c] = __fmaf_rn(a[e + 1][c], xb, y1[q][c]);
-                }
->>>>>>> Stashed changes
               }
             }
           }
@@ -551,16 +523,12 @@ __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, 
       if (wgx) {
         const float sum = warp_add_many<RB>(acc);
         const int row = lane / (32 / RB);
-<<<<<<< Updated upstream
         if (lane % (32 / RB) == 0 && row < nb) {
           if (pairs)
             add_pair(rw + jb + row, sum);
           else
             rw[jb + row] = sum;
         }
-=======
-        if (lane % (32 / RB) == 0 && row < nb) add_pair(rw[jb + row], sum);
->>>>>>> Stashed changes
         __syncwarp();
       }
     }
@@ -579,11 +547,7 @@ __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, 
     for (int j = t; j < nk; j += kBBT) {
       KahanF32 sum;
 #pragma unroll
-<<<<<<< Updated upstream
       for (int w = 0; w < kBBT / 32; w++) add_pair(sum, red + w * kFusedRows + j, pairs);
-=======
-      for (int w = 0; w < kBBT / 32; w++) add_pair(sum, red[w * kFusedRows + j]);
->>>>>>> Stashed changes
       dst[j] = sum.value();
     }
     finish_gx(it, items, cnt, partials, flag);
@@ -595,7 +559,7 @@ __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, 
 // the columns j of up to eight chunks (x_j and the column sums gx in
 // registers), a warp walks eight rows at a time and reduces their sums y.
 __device__ void blk_rows_fused(const BItem& it, int64_t i0, int64_t i1, int ks, int items, int* cnt, float* partials,
-                               float2* red, int* flag) {
+                               float* red, int* flag) {
   constexpr int RB = 8, NC = kFusedRowMax / 32;
   const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
   const int nk = (int)it.nk;
@@ -606,7 +570,6 @@ __device__ void blk_rows_fused(const BItem& it, int64_t i0, int64_t i1, int ks, 
     xq[q] = ((wy || wgA) && q * 32 + lane < nk) ? __ldg(it.x + q * 32 + lane) : 0.0f;
     cs[q] = 0.0f;
   }
-<<<<<<< Updated upstream
   float* const cw = red + wid * kFusedRows + lane;  // the lane's column sums (pairs), folded every 64 rows
 #pragma unroll
   for (int q = 0; q < NC; q++) cw[q * 32] = cw[q * 32 + kErr] = 0.0f;
@@ -614,15 +577,6 @@ __device__ void blk_rows_fused(const BItem& it, int64_t i0, int64_t i1, int ks, 
 #pragma unroll
     for (int q = 0; q < NC; q++) {
       add_pair(cw + q * 32, cs[q]);
-=======
-  float2* const cw = red + wid * kFusedRows + lane;  // the lane's column sums, folded every 64 rows
-#pragma unroll
-  for (int q = 0; q < NC; q++) cw[q * 32] = make_float2(0.0f, 0.0f);
-  auto fold = [&]() {
-#pragma unroll
-    for (int q = 0; q < NC; q++) {
-      add_pair(cw[q * 32], cs[q]);
->>>>>>> Stashed changes
       cs[q] = 0.0f;
     }
   };
@@ -682,11 +636,7 @@ __device__ void blk_rows_fused(const BItem& it, int64_t i0, int64_t i1, int ks, 
     for (int j = t; j < nk; j += kBBT) {
       KahanF32 sum;
 #pragma unroll
-<<<<<<< Updated upstream
       for (int w = 0; w < kBBT / 32; w++) add_pair(sum, red + w * kFusedRows + j, true);
-=======
-      for (int w = 0; w < kBBT / 32; w++) add_pair(sum, red[w * kFusedRows + j]);
->>>>>>> Stashed changes
       dst[j] = sum.value();
     }
     finish_gx(it, items, cnt, partials, flag);
@@ -698,7 +648,7 @@ __global__ void __launch_bounds__(kBBT, kBBlocksPerSM) tvc_batched_kernel(const 
                                                            const WItem* __restrict__ work, int nwork, int* counter,
                                                            int* gx_counters, float* gx_partials) {
   __shared__ int slot;
-  __shared__ float2 red[(kBBT / 32) * kFusedRows];
+  __shared__ float red[(kBBT / 32) * kFusedRows];
   __shared__ __align__(16) float xsm[kFusedRows];
   __shared__ int last_flag;
   for (int w = grab(counter, &slot); w < nwork; w = grab(counter, &slot)) {
@@ -726,7 +676,7 @@ __global__ void __launch_bounds__(kBBT, kBBlocksPerSM) tvc_batched_kernel(const 
     } else if (wi.kind == 4)
       blk_rows_fused(it, wi.a0, wi.a1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, &last_flag);
     else if (wi.kind == 1 || wi.kind == 5)
-      blk_gx_rect(it, wi.kind == 5 ? it.gA : nullptr, wi.a0, wi.a1, wi.c0, wi.c1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, &red[0].x, &last_flag);
+      blk_gx_rect(it, wi.kind == 5 ? it.gA : nullptr, wi.a0, wi.a1, wi.c0, wi.c1, wi.e0, wi.e1, gx_counters + wi.b, gx_partials, red, &last_flag);
     else
       blk_gA(it.gy, it.x, it.gA, it.nk, it.v, wi.a0, wi.a1, wi.c0, wi.c1);
   }
