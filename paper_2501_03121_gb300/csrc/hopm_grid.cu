@@ -184,13 +184,17 @@ __device__ void hg_tile(HgPhase& f) {
   int cost = INT32_MAX;
   for (int m = m0; m < m0 + 6; m++) {
     const int w = max(1, (n + m - 1) / m);
-    const int P = max(Pmin, min(16, min(kHgT / w, (f.nk + 3) / 4)));
-    const int c = m * ((f.nk + P - 1) / P + 4);  // a chunk costs about four more rows
-    if (c < cost) {
-      cost = c;
-      f.m = m;
-      f.w = w;
-      f.P = P;
+    // Phases: up to 16, more for long contracted modes (in rows: four for a
+    // chunk, one for eight phases' sums).
+    for (int p = 16; p <= 128; p *= 2) {
+      const int P = max(Pmin, min(p, min(kHgT / w, (f.nk + 3) / 4)));
+      const int c = m * ((f.nk + P - 1) / P + 4 + (P > 16 ? P / 8 : 0));
+      if (c < cost) {
+        cost = c;
+        f.m = m;
+        f.w = w;
+        f.P = P;
+      }
     }
     if (w <= 8) break;
   }
@@ -589,6 +593,19 @@ bool hopm_grid_wanted(int order, const int64_t* dims, tvc_dtype dt) {
   return sum <= kHgMaxVec && rest2 * es >= 64;
 }
 
+// Blocks of a run: one per SM for the larger tensors, fewer for those whose
+// phases are then mostly barrier, so that runs on several streams share the GPU
+// (a block fills its SM).  us per sweep alone / eight runs at once, one block
+// per SM -> this rule: FP64 16^3 23.6 / 23.0 -> 20.6 / 2.7, 32^3 27.8 / 27.2 -> 22.9
+// / 3.0, 64^3 25.5 / 24.8 -> 25.8 / 12.6; FP32 32^3 21.0 / 20.3 -> 17.6 / 2.3, 64^3
+// 19.8 / 19.0 -> 19.9 / 2.6, 100^3 21.5 / 21.1 -> 21.3 / 9.  (Queued kernels, captured,
+// alone / eight at once: FP64 16^3 42 / 6.3, 64^3 70 / 10, 128^3 79 / 13 against 31 /
+// 31 here, which still takes the whole GPU.)
+static int hg_blocks(int64_t N, tvc_dtype dt) {
+  const int64_t per = dt == TVC_F64 || dt == TVC_F32D ? 3500 : 16000;  // elements
+  return (int)std::min<int64_t>(device_sms(), std::max<int64_t>(16, (N + per - 1) / per));
+}
+
 // Bytes of its partial sums and barrier word (beside T and W_j).
 size_t hopm_grid_ws_bytes(int order, const int64_t* dims, tvc_dtype dt) {
   int64_t n = 1;
@@ -603,11 +620,12 @@ tvc_status hopm_grid_launch(const void* A, int order, const int64_t* dims, void*
   a.A = A;
   a.d = order;
   a.iters = iters;
-  int64_t n = 1;
+  int64_t n = 1, N = 1;
   for (int m = 0; m < order; m++) {
     a.dims[m] = dims[m];
     a.x[m] = x[m];
     n = std::max(n, dims[m]);
+    N *= dims[m];
   }
   a.scales = scales;
   a.tol = tol;
@@ -615,7 +633,7 @@ tvc_status hopm_grid_launch(const void* A, int order, const int64_t* dims, void*
   a.sweeps_out = sweeps_out;
   a.status_out = status_out;
   a.lam_hist = lam_hist;
-  const int blocks = device_sms();
+  const int blocks = hg_blocks(N, dt);
   a.arrived = static_cast<unsigned*>(ws);
   const size_t part = align_up((size_t)(n + blocks + 1) * vec_size(dt), 256);
   a.parts[0] = static_cast<char*>(ws) + 256;
