@@ -1,6 +1,6 @@
 // Power methods over many independent FP32 tensors of uneven order and
 // shape in one persistent launch: one thread-block cluster runs every sweep
-// of one tensor (largest tensors first, pulled from an atomic counter), its
+// of one tensor (small tensors: one block, batched_hopm_block.cu) (largest tensors first, pulled from an atomic counter), its
 // blocks meeting at the hardware cluster barrier.
 //
 // A sweep reads A twice and meets d cluster barriers:
@@ -44,14 +44,7 @@ constexpr int kHW = kHT / kWarp;      // warps per block
 constexpr int kHSlots = kHW;           // thread partials held per reduction (one warp reduces each)
 constexpr int kHXCap = 3072;          // vector entries held in shared memory
 
-struct HItem {
-  const float* A;
-  int d;
-  int64_t dims[TVC_MAX_ORDER];
-  float* x[TVC_MAX_ORDER];
-  double* lam;
-  int* status;
-};
+using HItem = HopmItem;
 
 // Column tiling of one pass for one block: m chunks of w columns, P rows at a time.
 struct HTile {
@@ -546,10 +539,48 @@ struct HLayout {
   size_t off_counter = 0, off_slots = 0, off_items = 0, off_scratch = 0, total = 0;
   HScratch sc{};
   int clusters = 0;
+  bool block = false;             // one block per tensor
+  int64_t slen = 0, zlen = 0;     // its scratch
 };
+
+// Batches of small tensors run one block per tensor (batched_hopm_block.cu): all
+// tensors of at most 65536 elements, or 64 or more of at most 220000; matrices of
+// at most 10000, or 32 or more of at most 40000.  ms of 5 sweeps, blocks /
+// clusters: 4096 of 3..6 per mode 0.86 / 2.9, 512 of 8..32 0.19 / 0.92, 4096 of 30..60
+// 3.3 / 6.7, 64 of 30..60 0.29 / 0.34; beyond the line one of 48^3 0.16 / 0.13, 64 of
+// 64^3 0.60 / 0.33, 8 matrices of 20..200 0.12 / 0.09 (64 of them 0.19 / 0.43), 304 of
+// 100..500 1.0 / 0.57.
+bool block_wanted(const hopm_batch_desc* d, int count) {
+  for (int b = 0; b < count; b++) {
+    int64_t N = 1;
+    for (int m = 0; m < d[b].order; m++) N *= d[b].dims[m];
+    const bool matrix = d[b].order == 2;
+    if (N > (matrix ? 10000 : 65536) && (count < (matrix ? 32 : 64) || N > (matrix ? 40000 : 220000))) return false;
+  }
+  return true;
+}
 
 HLayout layout_hopm(const hopm_batch_desc* d, int count) {
   HLayout L;
+  L.off_slots = 256;
+  if (block_wanted(d, count)) {
+    L.block = true;
+    for (int b = 0; b < count; b++) {
+      int64_t N = 1, least = d[b].dims[0];
+      for (int m = 0; m < d[b].order; m++) {
+        N *= d[b].dims[m];
+        least = std::min(least, d[b].dims[m]);
+        L.zlen = std::max(L.zlen, d[b].dims[m]);
+      }
+      L.slen = std::max(L.slen, N / least);
+    }
+    L.slen = (int64_t)align_up((size_t)L.slen, 64);
+    L.zlen = (int64_t)align_up((size_t)L.zlen, 64);
+    L.off_items = L.off_slots;
+    L.off_scratch = L.off_items + align_up((size_t)std::max(1, count) * sizeof(HItem), 256);
+    L.total = L.off_scratch + hopm_block_ws_bytes(L.slen, L.zlen);
+    return L;
+  }
   int64_t slen = 1, zlen = 1, xlen = 0, total = 0, largest = 1;
   for (int b = 0; b < count; b++) {
     int64_t N = 1, sum = 0;
@@ -578,11 +609,10 @@ HLayout layout_hopm(const hopm_batch_desc* d, int count) {
   while (cl > 2 && 1.25 * (double)largest * (blocks / (cl / 2)) < (double)total) cl /= 2;
   L.sc.cl = cl;
   L.clusters = std::max(1, std::min(count, blocks / cl));
-  L.off_slots = 256;
   L.off_items = L.off_slots + align_up((size_t)L.clusters * 2 * sizeof(int), 256);
   L.off_scratch = L.off_items + align_up((size_t)std::max(1, count) * sizeof(HItem), 256);
   L.total = L.off_scratch + (size_t)L.clusters *
-                                (2 * L.sc.slen + cl * (2 * L.sc.zlen + L.sc.xlen)) * sizeof(float);
+                                (2 * L.sc.slen + cl * (2 * L.sc.zlen + L.sc.xlen)) * sizeof(float) + 16;
   return L;
 }
 
@@ -655,6 +685,13 @@ extern "C" tvc_status hopm_batched(const hopm_batch_desc* descs, int count, int 
       return TVC_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return TVC_ERR_CUDA;
   }
+  if (L.block) {
+    cudaMemsetAsync(w + L.off_counter, 0, sizeof(int), st);
+    count_launches(1);
+    return cuda_status(hopm_block_launch(reinterpret_cast<const HItem*>(w + L.off_items), count, iters,
+                                         reinterpret_cast<int*>(w + L.off_counter),
+                                         reinterpret_cast<float*>(w + L.off_scratch), L.slen, L.zlen, st));
+  }
   if (prepare_kernel() != cudaSuccess) return cuda_status(cudaGetLastError());
   cudaMemsetAsync(w + L.off_counter, 0, sizeof(int), st);
   cudaLaunchConfig_t cfg{};
@@ -670,7 +707,8 @@ extern "C" tvc_status hopm_batched(const hopm_batch_desc* descs, int count, int 
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   HScratch sc = L.sc;
-  sc.base = reinterpret_cast<float*>(w + L.off_scratch);
+  // vectors in memory are read in 16-byte pieces, whatever the workspace's own alignment
+  sc.base = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(w + L.off_scratch) + 15) & ~(uintptr_t)15);
   const cudaError_t e =
       cudaLaunchKernelEx(&cfg, hopm_batched_kernel, reinterpret_cast<const HItem*>(w + L.off_items), count, iters,
                          reinterpret_cast<int*>(w + L.off_counter), reinterpret_cast<int*>(w + L.off_slots), sc);

@@ -76,6 +76,20 @@ tvc_status hopm_grid_launch(const void* A, int order, const int64_t* dims, void*
 // Sticky error word of its grid barrier (cleared when clear != 0).
 tvc_status hopm_grid_device_error(int* code_out, int clear);
 
+// One tensor of a batch of power methods, and the kernel that runs one block per
+// tensor (batched_hopm_block.cu): slen >= N / min(dims), zlen >= max(dims) floats.
+struct HopmItem {
+  const float* A;
+  int d;
+  int64_t dims[TVC_MAX_ORDER];
+  float* x[TVC_MAX_ORDER];
+  double* lam;
+  int* status;
+};
+size_t hopm_block_ws_bytes(int64_t slen, int64_t zlen);
+cudaError_t hopm_block_launch(const HopmItem* items, int count, int iters, int* counter, float* scratch, int64_t slen,
+                              int64_t zlen, cudaStream_t st);
+
 // 1D split over virtual ranks (split.cu).  check_split validates parts,
 // starts and s against the tensor; slab_dims gives rank r's dims.
 tvc_status check_split(int parts, const int64_t* starts, int order, const int64_t* dims, int s);
