@@ -10,7 +10,8 @@
 // wants gx and another of its results, one item computes all of them for a
 // range of columns (v >= 32) or rows (v == 1) from one read of A; the other
 // cases have an item kind per result.  gx items of one tensor leave partial
-// sums that the tensor's last item adds in a fixed order.  With TVC_BATCH_PREUPLOADED the descriptors of a previous call are reused and a
+// sums that the tensor's last item adds in a fixed order.  With
+// TVC_BATCH_PREUPLOADED the descriptors of a previous call are reused and a
 // call issues only a memset and one kernel, so it can be captured in a CUDA
 // graph and replayed.
 //
@@ -459,7 +460,10 @@ __device__ void blk_cols_fused(const BItem& it, int64_t c0, int64_t c1, int ks, 
   if (wy || wgA)
     for (int j = t; j < nk; j += kBBT) xsm[j] = __ldg(it.x + j);
   if (wgx)
-    for (int j = lane; j < (pairs ? kErr + nk : nk); j += 32) rw[j] = 0.0f;
+    for (int j = lane; j < nk; j += 32) {
+      rw[j] = 0.0f;
+      if (pairs) rw[kErr + j] = 0.0f;
+    }
   __syncthreads();
   const int nbat = (nk + RB - 1) / RB, per = (nk + nbat - 1) / nbat;
   for (int64_t g = c0 + wid * 128; g < c1; g += (kBBT / 32) * 128) {
@@ -725,10 +729,15 @@ int64_t item_elems(const std::vector<BItem>& items) {
 
 // The fused item kind of a tensor (3: columns, 4: rows; 0: none): where one
 // read of A serves gx and another result, or gx alone in the column case.
+// Without gx nothing is shared (y reads A, gA does not), and separate items are
+// faster: y and gA of 512 matrices of 20..200 per mode 111 us fused, 32 apart; of
+// 4096 of 100..500 1321 / 654.  Neither do tiny tensors gain: all three results
+// of 4096 of 4..12 per mode 81 / 49 us, of 8..16 84 / 68, of 16..24 139 / 146; gx of
+// 8..16 39 / 43.
 int fused_kind(const BItem& it) {
-  const int wanted = (it.y != nullptr) + (it.gx != nullptr) + (it.gA != nullptr);
-  if (it.v >= kGxWarpRows && it.nk <= kFusedRows && (it.gx || wanted > 1)) return 3;
-  if (it.v == 1 && it.nk >= kFusedRowMin && it.nk <= kFusedRowMax && wanted > 1) return 4;
+  if (!it.gx || it.u * it.nk * it.v < (it.y && it.gA ? 4000 : 1000)) return 0;
+  if (it.v >= kGxWarpRows && it.nk <= kFusedRows) return 3;
+  if (it.v == 1 && it.nk >= kFusedRowMin && it.nk <= kFusedRowMax && (it.y || it.gA)) return 4;
   return 0;
 }
 
