@@ -656,41 +656,50 @@ __global__ void __launch_bounds__(kTmcThreads) tmc_rows_group_kernel(const TmcAr
   }
 }
 
-// Y[o] = alpha * sum_s partial[s][o] + beta * Y[o]: a block adds 32 outputs,
-// each of its 8 warps a contiguous share of the splits in order, then the
-// warps in order (FP32 compensated).
+// Sum of partial results: compensated in FP32.
+template <class W>
+struct TmcSum : KahanF32 {};
+template <>
+struct TmcSum<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+
+// Y[o] = alpha * sum_s partial[s][o] + beta * Y[o], s ascending.
 template <class W>
 __global__ void __launch_bounds__(256) tmc_reduce_kernel(const W* __restrict__ partial, W* __restrict__ Y, int64_t n,
                                                          int splits, double alpha, double beta) {
+  for (int64_t o = (int64_t)blockIdx.x * 256 + threadIdx.x; o < n; o += (int64_t)gridDim.x * 256) {
+    TmcSum<W> s;
+    for (int k = 0; k < splits; k++) s.add(partial[(int64_t)k * n + o]);
+    W r = (W)alpha * s.value();
+    if (beta != 0.0) r += (W)beta * Y[o];
+    Y[o] = r;
+  }
+}
+
+// The same for few outputs and many splits: a block adds 32 outputs, each of its
+// 8 warps a contiguous share of the splits in order, then the warps in order.
+template <class W>
+__global__ void __launch_bounds__(256) tmc_reduce_many_kernel(const W* __restrict__ partial, W* __restrict__ Y, int64_t n,
+                                                         int splits, double alpha, double beta) {
   __shared__ W sums[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  using Sum = std::conditional_t<sizeof(W) == 8, double, KahanF32>;
-  auto add = [](Sum& t, W v) {
-    if constexpr (sizeof(W) == 8)
-      t += v;
-    else
-      t.add(v);
-  };
-  auto value = [](const Sum& t) -> W {
-    if constexpr (sizeof(W) == 8)
-      return t;
-    else
-      return t.value();
-  };
   for (int64_t o0 = (int64_t)blockIdx.x * 32; o0 < n; o0 += (int64_t)gridDim.x * 32) {
     const int64_t o = o0 + lane;
-    Sum s{};
+    TmcSum<W> s;
     if (o < n) {
 #pragma unroll 8
-      for (int k = splits * w / 8; k < splits * (w + 1) / 8; k++) add(s, partial[(int64_t)k * n + o]);
+      for (int k = splits * w / 8; k < splits * (w + 1) / 8; k++) s.add(partial[(int64_t)k * n + o]);
     }
     __syncthreads();  // the previous outputs' sums are read
-    sums[w][lane] = value(s);
+    sums[w][lane] = s.value();
     __syncthreads();
     if (w == 0 && o < n) {
-      Sum t{};
-      for (int k = 0; k < 8; k++) add(t, sums[k][lane]);
-      W r = (W)alpha * value(t);
+      TmcSum<W> t;
+      for (int k = 0; k < 8; k++) t.add(sums[k][lane]);
+      W r = (W)alpha * t.value();
       if (beta != 0.0) r += (W)beta * Y[o];
       Y[o] = r;
     }
@@ -717,14 +726,31 @@ int tmc_rp(tvc_dtype dt, int64_t R) {
   return 16;
 }
 
-// Whether the register-blocked kernels take the shape: FP32 accumulation,
-// where neither the copy pipelines for up to eight rows of X (p.async,
-// p.group) nor very short rows apply; columns against up to four rows of X
-// are bound by loads and stay with the one-element kernel (96x3935x409 FP32,
-// R = 4, mode 2 of the MTTKRP: 193 us, 214 here).
+// Whether the register-blocked kernels take the shape: FP32 accumulation, where
+// neither the copy pipelines for up to eight rows of X (p.async, p.group) nor
+// very short rows apply, and where their blocks fill the GPU: a block of columns
+// covers four times the outputs of the one-element kernel's, which is up to
+// three times faster on fewer.  On 1084 shapes of 1e3..2e8 elements, R 2..33, the
+// rule is within 1.3% of the faster of the two (register-blocked wherever it
+// could run: 39% off).  us, one-element / register-blocked: rows (v == 1) 14x14
+// R = 13 1.9 / 2.6, 400x200 R = 16 6.0 / 3.9; columns 39x1487x59 BF16 R = 12 23.9 / 62.1,
+// 315x174x81 BF16 R = 6 15.5 / 56.3, 1x385x18 R = 9 8.5 / 4.9, 485x72x1900 F16 R = 16 195
+// / 120, 1160x2362x33 F32 R = 6 109 / 192, 353x64x6392 E4M3 R = 5 128 / 86, 435342x2x69 F32
+// R = 13 746 / 994.
 bool simt_wanted(const TmcPlan& p, const Shape& s, tvc_dtype dt, int64_t R) {
-  return vec_size(dt) == 4 && !p.async && !p.group && (s.v == 1 ? s.nk >= 4 : s.v >= 4 && R > 4) &&
-         tmc_simt_blocks(s.u, s.v) * ((R + 3) / 4) <= 0x7FFFFFFF;  // one grid dimension
+  if (vec_size(dt) != 4 || p.async || p.group) return false;
+  const int rp = tmc_simt_rp(R);
+  const int64_t blocks = tmc_simt_blocks(s.u, s.v) * ((R + rp - 1) / rp), sms = device_sms();
+  if (blocks > 0x7FFFFFFF) return false;  // one grid dimension
+  if (s.v == 1) {
+    if (dt == TVC_F32 && R > 4 && R <= 8 && s.u < 512) return false;
+    return s.nk >= 64 || (s.nk >= 32 && s.u >= 128);
+  }
+  if (s.v < 4 || R <= 4) return false;  // bound by loads: the one-element kernel
+  if (s.uv < 128) return s.nk >= 128 && (R > 8 || s.nk < 8192);  // phases of rows within a block
+  if (R <= 8) return dt != TVC_F32 && blocks >= 3 * sms && s.nk >= 8;
+  return (blocks >= 27 * sms && s.nk >= 3) || (blocks >= 8 * sms && s.nk >= 8) || (blocks >= 4 * sms && s.nk >= 16) ||
+         blocks * (s.nk / 256) >= 256;  // with n_k split
 }
 
 // A == nullptr (the workspace query) plans for a 16-byte aligned A; the
@@ -897,9 +923,14 @@ tvc_status run(const void* A, const Shape& s, const void* X, int64_t R, void* Y,
   int launches = 1;
   if (p.splits > 1) {
     const int64_t n = s.uv * R;
-    const int blocks = (int)std::min<int64_t>((n + 31) / 32, 64LL * device_sms());
-    tmc_reduce_kernel<W><<<blocks, 256, 0, st>>>(static_cast<const W*>(ws), static_cast<W*>(Y), n, p.splits, alpha,
-                                                 beta);
+    // 440000 outputs of 2 splits 11 us with a warp per share, 3 with a thread per output
+    if (p.splits >= 8 && n <= 32 * 1024) {
+      tmc_reduce_many_kernel<W><<<(int)((n + 31) / 32), 256, 0, st>>>(static_cast<const W*>(ws), static_cast<W*>(Y), n,
+                                                                      p.splits, alpha, beta);
+    } else {
+      const int blocks = (int)std::min<int64_t>((n + 255) / 256, 8LL * device_sms());
+      tmc_reduce_kernel<W><<<blocks, 256, 0, st>>>(static_cast<const W*>(ws), static_cast<W*>(Y), n, p.splits, alpha, beta);
+    }
     launches++;
   }
   count_launches(launches);
