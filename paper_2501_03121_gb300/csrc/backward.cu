@@ -8,6 +8,8 @@
 // gx, v == 1 and k > 0: gx = (A viewed as u x n_k) x_0 gy, i.e. a TVC of
 //   mode 0 on the unfolded view (the column kernel), with gy times the slab
 //   scale for narrow storage.
+// gx, FP32 arithmetic, mode 0 with rows of at most 512 bytes: gx = (A viewed as n_k x v) x_1 gy, a
+//   TVC of the last mode (the row kernels).
 // gx, otherwise: each thread owns 16-byte pieces of columns (i, l), keeps
 //   their gy in registers (FP64 arithmetic: in shared memory) and streams the piece's rows, eight (rows off 16-byte
 //   boundaries: four) in flight; a warp reduces the rows' dot products over
@@ -563,12 +565,13 @@ __global__ void __launch_bounds__(256) tvc_gradA_slab_kernel(const V* __restrict
 namespace {
 
 struct GxPlan {
-  bool via_tvc = false;  // v == 1
+  bool via_tvc = false;   // v == 1
+  bool via_rows = false;  // mode 0, short rows
   int rch = 8;        // rows per chunk
   bool al = false;    // rows of A on 16-byte boundaries
   int64_t nchunks = 1, nblk = 1, pps = 1;
   size_t ws_partial = 0, ws_gy = 0, ws_tvc = 0, total = 0;
-  Shape view;  // v == 1: (u, nk) mode 0
+  Shape view;  // via_tvc: (u, nk) mode 0; via_rows: (nk, v) mode 1
 };
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
@@ -591,6 +594,18 @@ GxPlan plan_gx(const Shape& s, tvc_dtype dt, const void* A) {
   const int64_t es = (int64_t)elem_size(dt);
   g.al = (s.v * es) % 16 == 0 && aligned(A, 16);
   g.pps = cdiv(s.v * es, 16);
+  if (s.mode == 0 && g.pps <= 32 && vs == 4) {
+    // short rows of a matrix n_k x v: gx = rows . gy, a TVC of its last mode (a
+    // block here would keep a few lanes busy: 261039 entries of order one E4M3
+    // 296 us, 16409x17 BF16 19)
+    g.via_rows = true;
+    const int64_t d2[2] = {s.nk, s.v};
+    make_shape(2, d2, 1, &g.view);
+    for (uintptr_t al = elem_size(dt); al <= 256; al *= 2)
+      g.ws_tvc = std::max(g.ws_tvc, tvc_ws_bytes(g.view, dt, reinterpret_cast<const void*>(al)));
+    g.total = g.ws_tvc;
+    return g;
+  }
   // One wave of blocks: chunks of 256 rows, or fewer (down to 32) where the
   // pieces alone do not fill it.
   const int64_t wave = (int64_t)device_sms() * (dt == TVC_E4M3 ? kGxBlocks<TVC_E4M3> : kGxBlocks<TVC_F32>);
@@ -615,6 +630,24 @@ GxPlan plan_gx(const Shape& s, tvc_dtype dt, const void* A) {
       g.rch = kGx64Rows;
       g.nchunks = cdiv(s.nk, g.rch);
       g.nblk = 1;
+    }
+  } else if (tiles < wave) {
+    // few pieces: the cut of the rows with the shortest time, in rows of 256
+    // pieces (a block costs about 16 beside its own), down to eight rows
+    // (130x260 E4M3 mode 0 11 -> 5 us)
+    double cost = 0.0;
+    const int64_t n0 = cdiv(s.nk, kGxRows), n1 = cdiv(s.nk, 8);
+    for (int64_t n = n0;; n = std::min(n1, std::max(n + 1, n * 5 / 4))) {
+      const int64_t rch = cdiv(cdiv(s.nk, n), 8) * 8, nch = cdiv(s.nk, rch);
+      const int64_t nblk = std::max<int64_t>(1, std::min(tiles, wave / nch));
+      const double c = (double)(cdiv(tiles, nblk) * rch + 16) * (double)std::max<int64_t>(1, cdiv(nch * nblk, wave));
+      if (n == n0 || c < cost) {
+        cost = c;
+        g.rch = (int)rch;
+        g.nchunks = nch;
+        g.nblk = nblk;
+      }
+      if (n == n1) break;
     }
   } else {
     g.nchunks = std::max(cdiv(s.nk, kGxRows), std::min(cdiv(s.nk, 32), wave / tiles));
@@ -665,6 +698,7 @@ tvc_status grad_x(const Shape& s, const void* A, const void* gy, void* gx, tvc_d
                   void* ws, size_t ws_bytes, cudaStream_t st) {
   const GxPlan g = plan_gx(s, dt, A);
   if (g.total > 0 && (ws == nullptr || ws_bytes < g.total)) return TVC_ERR_WORKSPACE;
+  if (g.via_rows) return tvc_launch(A, g.view, gy, gx, dt, scales, 1.0, 0.0, ws, g.ws_tvc, st);
   if (g.via_tvc) {
     char* w = static_cast<char*>(ws);
     const void* gyv = gy;
