@@ -1636,10 +1636,33 @@ static bool plan_slab_tile(Plan& p, const Shape& s, tvc_dtype dt, int sms) {
 
 // Rows (v == 1) off 16-byte boundaries that go to the ragged row kernel: of
 // at least 16 bytes (shorter ones measured no faster there), but for FP32
-// rows of 13 to 15 elements (staged 3920 GB/s, here 3706).
-static bool rows_ragged_wanted(int64_t nk, size_t es) {
-  const int64_t bytes = nk * (int64_t)es;
-  return bytes >= 16 && !(es == 4 && bytes > 48 && bytes < 64);
+// rows of 13 to 15 elements (staged 3920 GB/s, here 3706); from 128 bytes on
+// only in tensors large enough that its few long chains of loads are covered.
+// Staged or plain rows / here, us: BF16 2000x300 4.1 / 5.6, 40000x300 15 / 8.3; E4M3
+// 1851x534 4.5 / 7.6; F32 739x655 3.6 / 5.8, 100000x101 18 / 12, 30000x979 35 / 29 (within
+// 5% of the faster of the two on 500 shapes; up to 2.6x slower without the sizes).
+// vb: bytes that the plain kernels load at a time.
+static bool rows_ragged_wanted(const Shape& s, size_t es, int vb) {
+  const int64_t row = s.nk * (int64_t)es, bytes = s.u * row;
+  if (row < 16 || (es == 4 && row > 48 && row < 64)) return false;
+  if (row < 128) return vb < 4 || bytes >= 1000000;
+  if (es == 4) return bytes >= (row < 1024 ? 8000000 : 64000000);
+  if (es == 1) return bytes >= 8000000;
+  return row >= 4096 || bytes >= (row < 1024 ? 8000000 : 16000000);
+}
+
+// Columns (v >= 32) off 16-byte boundaries that go to the ragged column kernel:
+// a thread there takes 16 bytes of a row where the plain one takes one or two
+// elements, so it wants enough pieces (T) or enough rows to split.  Element
+// loads / here, us: BF16 8x129x84 4.6 / 7.4, 16x12x40x592 mode 0 4.3 / 8.3, 3x700x24321 24 /
+// 14, 5x300x60001 43 / 26; E4M3 9x126x4332 mode 0 3.6 / 7.8; F32 2x40x50001 5.8 / 7.0.
+static bool cols_ragged_wanted(const Shape& s, tvc_dtype dt, int vb, int sms) {
+  const int64_t T = s.u * ceil_div(s.v * (int64_t)elem_size(dt), 16);
+  if (T >= (int64_t)sms * 1280) return true;
+  if (dt == TVC_E4M3 && vb >= 4) return false;  // 1664x56440 mode 0 25 us, 32 here
+  if (s.nk >= 512 && T >= (int64_t)sms * (dt == TVC_F32 ? 64 : 20)) return true;
+  if (s.nk >= 128 && T >= (int64_t)sms * 64) return true;
+  return dt != TVC_F32 && s.nk >= 32 && T >= (int64_t)sms * 128;
 }
 
 static void plan_rows_ragged(Plan& p, const Shape& s, size_t es, int sms) {
@@ -1676,12 +1699,10 @@ static void plan_rows_ragged(Plan& p, const Shape& s, size_t es, int sms) {
 // 9.0 -> 5.1 us, BF16 10.5 -> 4.6, E4M3 13.4 -> 4.0; 300x70x33 FP64 12.9 ->
 // 7.3).  Between the two the column kernels stream longer runs per thread and
 // stay faster (FP32 1000x1000x100 mode 0 68 us, phased 110; 16 MB FP64 10.5,
-// phased 12.7).
+// phased 12.7; 16846x4441 single-double mode 0 109, phased 183).
 // The workspace stays at least what the column kernels would take, so that
 // callers who lend a fixed scratch keep the limits they had.
-// FP64 up to 18 MB: 128^3 takes the same 10.5 us on the device, but one launch
-// and no scratch in place of three, which is what a caller waits for.
-constexpr int64_t kPhasedSmall = 12 << 20, kPhasedSmallF64 = 18 << 20;
+constexpr int64_t kPhasedSmall = 12 << 20;
 
 static void set_phased(Plan& p, const Shape& s, tvc_dtype dt, const void* A, int w, int64_t splits) {
   const int64_t es = (int64_t)elem_size(dt);
@@ -1697,11 +1718,18 @@ static void set_phased(Plan& p, const Shape& s, tvc_dtype dt, const void* A, int
 
 // Few outputs (v > 1) over many rows: the widest block of pieces that the
 // outputs fill, the rows split over one wave of blocks (1000000x64 mode 0:
-// FP64 949 -> 115 us, FP32 684 -> 46, E4M3 831 -> 33; 8388608x128: FP32 1158
-// -> 610, BF16 2740 -> 375).
+// FP64 949 -> 115 us, FP32 684 -> 46, E4M3 831 -> 22; 8388608x128: FP32 1158
+// -> 610, BF16 2740 -> 375).  Up to 16 pieces from 4 MB on; up to 64 from 16 MB on,
+// or from 4 MB in FP64 arithmetic, on 16-byte boundaries (narrow storage off
+// them too); on 600 shapes beyond that the column and slab kernels were faster,
+// by up to 3.6x on small ones.
 static bool plan_phased_few(Plan& p, const Shape& s, tvc_dtype dt, const void* A, int sms) {
-  const int64_t pieces = s.u * ceil_div(s.v * (int64_t)elem_size(dt), 16);
-  if (pieces > 16 * sms || s.nk < 4096) return false;
+  const int64_t es = (int64_t)elem_size(dt), pieces = s.u * ceil_div(s.v * es, 16), bytes = s.N * es;
+  if (pieces > 64 || s.nk < 4096 || bytes < (4 << 20)) return false;
+  if (pieces > 16) {
+    const bool f64 = vec_size(dt) == 8, al = (s.v * es) % 16 == 0 && aligned(A, 16);
+    if (!(al ? f64 || bytes >= (16 << 20) : es < 4 && bytes >= (16 << 20))) return false;
+  }
   int w = 1;
   while (w < kThreads && w < pieces) w *= 2;
   const int64_t blocks = (int64_t)sms * phased_blocks_per_sm(dt);
@@ -1717,7 +1745,11 @@ static void plan_cols_phased(Plan& p, const Shape& s, tvc_dtype dt, const void* 
   const int64_t blocks = (int64_t)sms * phased_blocks_per_sm(dt);
   int64_t splits = 1;
   int w = 8;
-  if (s.N * es <= kPhasedSmall && s.nk >= 8) {
+  // Short modes leave the phases nothing to share: 6x13x26x14x3 E4M3 mode 1 3.3 us,
+  // phased 6.6.
+  const bool al = (s.v * es) % 16 == 0 && aligned(A, 16);
+  const int64_t least = es < 4 ? (al ? 32 : 16) : (al || dt == TVC_F64) ? 16 : 64;
+  if (s.N * es <= kPhasedSmall && s.nk >= least && pieces <= 10000) {
     w = 128;
     while (w > 8 && ceil_div(pieces, w) < blocks) w /= 2;
     while (s.nk * w < 4 * kThreads && w < 128) w *= 2;
@@ -1736,10 +1768,9 @@ static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool all
   const int64_t target_threads = (int64_t)sms * 2048;
   const int64_t S = s.nk * s.v;
   const size_t es = elem_size(dt);
-  // Rows off 16-byte boundaries (tvc_ragged.cu); FP32 columns only where the
-  // pieces give enough threads (64x264x475 mode 1: 8.5 us, element loads 7.5).
-  const bool ragged = dt != TVC_F64 && dt != TVC_F32D && pick_vec(dt, s.v == 1 ? s.nk : s.v, A) * (int)es < 16 &&
-                      !(dt == TVC_F32 && s.v >= 32 && s.u * ceil_div(s.v, 4) < (int64_t)sms * 64);
+  // Rows off 16-byte boundaries (tvc_ragged.cu).
+  const int vb = pick_vec(dt, s.v == 1 ? s.nk : s.v, A) * (int)es;
+  const bool ragged = dt != TVC_F64 && dt != TVC_F32D && vb < 16 && (s.v < 32 || cols_ragged_wanted(s, dt, vb, sms));
   if (s.v >= 32) {
     p.kind = ragged ? K_COLS_RAGGED : K_COLS;
     p.vec = pick_vec(dt, s.v, A);
@@ -1764,7 +1795,7 @@ static Plan make_plan_impl(const Shape& s, tvc_dtype dt, const void* A, bool all
     plan_cols_phased(p, s, dt, A, sms);
   } else if (dt == TVC_F64 && aligned(A, 16) && s.v < 32 && plan_f64_tile(p, s, sms)) {
     // FP64 small slabs and short rows: the copy-engine tile kernel.
-  } else if (s.v == 1 && !f64acc && ragged && rows_ragged_wanted(s.nk, es)) {
+  } else if (s.v == 1 && !f64acc && ragged && rows_ragged_wanted(s, es, vb)) {
     plan_rows_ragged(p, s, es, sms);
   } else if (s.v == 1 && !f64acc && allow_staged && aligned(A, 16) &&
              s.nk <= 8 * 32 * (int64_t)pick_vec(dt, s.nk, A, 4) && s.u >= 8) {
