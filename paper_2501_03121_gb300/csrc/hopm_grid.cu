@@ -13,11 +13,11 @@
 // Parts and W buffers alternate between phases: a block writes one again
 // only after a barrier behind its last reader.
 //
-// Bound: latency; of the 13 us of a phase of FP64 128^3 (FP32: 9) the
-// contraction takes 6 (2.3), the barrier 2.7 (2), the parts 1.6 (0.8), norm and
-// x_j 2.7.  One block of 512 threads per SM: 1024 threads of 64 registers
-// measured 30-60% slower.  See hopm_grid_wanted for the line to the queued
-// kernels.
+// Bound: latency; about half of the 10.5 us of a phase of FP64 128^3 (FP32: 7)
+// is the contraction, the rest the barrier, the parts, norm and x_j.  One block of
+// 512 threads per SM: 1024 threads of 64 registers measured 30-60% slower.  See hopm_grid_wanted for the line to the queued
+// kernels.  A run of a tensor beyond a few MB fills the GPU (hg_blocks), so several
+// on different streams follow one another.
 #include <algorithm>
 #include <mutex>
 #include <set>
@@ -572,24 +572,31 @@ cudaError_t hg_launch(const HgArgs& a, int blocks, cudaStream_t st) {
 // of A that are at least four pieces long; and the sizes for which it pays:
 // beyond them the queued kernels, with more loads in flight per SM, win back
 // what their launches cost.  us per sweep, queued / here: FP64 128^3 (17 MB)
-// 121 / 39, 200x300x256 (123 MB) 144 / 97, 101x90x70x80 (407 MB) 309 / 280,
-// 301x257x311 (odd rows, 192 MB) 176 / 182; FP32 128^3 80 / 29, 301x257x311
-// (96 MB) 112 / 74, 101x90x70x80 (204 MB) 172 / 145, 400^3 (256 MB) 158 / 161;
-// BF16 301x257x311 (48 MB) 113 / 80, 101x90x70x80 (102 MB) 143 / 105, 400^3
-// (128 MB) 127 / 105, 989x197x570 (222 MB) 172 / 255; E4M3 400^3 (64 MB) 116 /
-// 63, 989x197x570 (111 MB) 145 / 176.
+// 121 / 32, 200x300x256 (123 MB) 144 / 97, 101x90x70x80 (407 MB) 309 / 280; FP32
+// 128^3 80 / 22, 400^3 (256 MB) 158 / 161; BF16 101x90x70x80 (102 MB) 143 / 105,
+// 400^3 (128 MB) 127 / 105, 989x197x570 (222 MB) 172 / 255; E4M3 400^3 (64 MB) 116 /
+// 63.  Rows off 16-byte boundaries pay up to three quarters of that but for E4M3
+// (425x12x101x77 FP32, 159 MB, 132 / 142; 112x192x487 FP64, 84 MB, 180 / 126), and T
+// and W_1 at most 12 MB (they are written and read by every sweep: 25x2x33x804x28 E4M3, 74 MB
+// of W_1, 277 / 353; 4x20x948x502 FP32, 38 MB, 196 / 248).
 bool hopm_grid_wanted(int order, const int64_t* dims, tvc_dtype dt) {
   if (order < 3) return false;
   const int64_t es = (int64_t)elem_size(dt);
-  const int64_t most = es >= 4 ? 160000000 : es == 2 ? 104000000 : 72000000;
+  int64_t most = es == 8 ? 160000000 : es >= 2 ? 104000000 : 72000000;
   int64_t N = 1, sum = 0, rest2 = 1;
+  for (int m = 2; m < order; m++) {
+    if (dims[m] > kHgMaxVec) return false;
+    rest2 *= dims[m];
+    if (rest2 > most) return false;
+  }
+  if (es > 1 && rest2 * es % 16 != 0) most = most / 4 * 3;
   for (int m = 0; m < order; m++) {
     if (dims[m] > kHgMaxVec) return false;
     N *= dims[m];
     if (N * es > most) return false;
-    if (m >= 2) rest2 *= dims[m];
     sum += (dims[m] + 3) / 4 * 4;
   }
+  if (N / std::min(dims[0], dims[1]) * (int64_t)vec_size(dt) > 12000000) return false;
   return sum <= kHgMaxVec && rest2 * es >= 64;
 }
 

@@ -39,11 +39,12 @@ def test_batched_gx_of_rows():
     assert bool((gx[1:] == n).all())
 
 
-@pytest.mark.parametrize("dims", [(2, 2, 2000, 1900), (3, 2, 1200, 1000)])
+@pytest.mark.parametrize("dims", [(2, 2, 1200, 1200), (2, 2, 1450, 1000)])
 def test_power_method_of_few_leading_entries(dims):
-    # z_0[0] = 2^25 + n - 1 and z_0[1] = n: their quotient, to the rounding of
-    # the two entries of x_0, of z_0[0], and of the tree over a block's threads
-    # (nine levels of half a spacing of 2^25, 18 of 3e7, in the first block).
+    # z_0[0] = 2^25 + n - 1 and z_0[1] = n: their quotient, to the rounding (2^-24
+    # each) of the two entries of x_0 and of z_0[0], and of the tree over a block's
+    # threads (nine levels of half a spacing of 2^25).  A plain chain loses one per
+    # product of the thread that holds the large one, about 37.
     n = dims[2] * dims[3]
     A = torch.ones(dims, device="cuda")
     A.view(-1)[0] = 2.0**25
@@ -56,4 +57,4 @@ def test_power_method_of_few_leading_entries(dims):
     assert tg.kernel_launches() - before == 1  # the one-launch kernel
     got = r.x[0][0].double().item() / r.x[0][1].double().item()
     want = (2.0**25 + n - 1) / n
-    assert abs(got - want) <= 6 * 2.0**-24 * want + 9 * 2 / n
+    assert abs(got - want) <= 3 * 2.0**-24 * want + 9 * 2 / n
