@@ -633,14 +633,14 @@ GxPlan plan_gx(const Shape& s, tvc_dtype dt, const void* A) {
     }
   } else if (tiles < wave) {
     // few pieces: the cut of the rows with the shortest time, in rows of 256
-    // pieces (a block costs about 16 beside its own), down to eight rows
+    // pieces (a tile costs about four beside its own, a block 16), down to eight rows
     // (130x260 E4M3 mode 0 11 -> 5 us)
     double cost = 0.0;
     const int64_t n0 = cdiv(s.nk, kGxRows), n1 = cdiv(s.nk, 8);
     for (int64_t n = n0;; n = std::min(n1, std::max(n + 1, n * 5 / 4))) {
       const int64_t rch = cdiv(cdiv(s.nk, n), 8) * 8, nch = cdiv(s.nk, rch);
       const int64_t nblk = std::max<int64_t>(1, std::min(tiles, wave / nch));
-      const double c = (double)(cdiv(tiles, nblk) * rch + 16) * (double)std::max<int64_t>(1, cdiv(nch * nblk, wave));
+      const double c = (double)(cdiv(tiles, nblk) * (rch + 4) + 16) * (double)std::max<int64_t>(1, cdiv(nch * nblk, wave));
       if (n == n0 || c < cost) {
         cost = c;
         g.rch = (int)rch;

@@ -64,54 +64,49 @@ __device__ __forceinline__ void fma2(u64& acc, u64 a, u64 b) {
 // one): the aligned words that hold it, and the cut.
 template <int BYTES>
 struct Window {
-  static constexpr int N = BYTES >= 4 ? BYTES / 4 : 1;
+  static_assert(BYTES >= 4 && BYTES <= 16, "four elements of 1, 2 or 4 bytes");
+  static constexpr int N = BYTES / 4;
   uint32_t w[2 * N];
 
   template <bool AL>
   __device__ __forceinline__ void load(uint64_t ad, int valid) {
-    if constexpr (BYTES == 2) {
-      const uint8_t* p = reinterpret_cast<const uint8_t*>(ad);
-      w[0] = __ldcs(p);
-      if (valid > 1) w[0] |= (uint32_t)__ldcs(p + 1) << 8;
-    } else {
-      const uint64_t lo = AL ? ad : ad & ~(uint64_t)(BYTES - 1);
-      const bool two = !AL && (int)(ad - lo) + valid > BYTES;
-      if constexpr (BYTES == 16) {
-        const uint4* p = reinterpret_cast<const uint4*>(lo);
-        const uint4 a = __ldcs(p);
-        w[0] = a.x;
-        w[1] = a.y;
-        w[2] = a.z;
-        w[3] = a.w;
-        if constexpr (!AL) {
-          const uint4 b = two ? __ldcs(p + 1) : make_uint4(0u, 0u, 0u, 0u);
-          w[4] = b.x;
-          w[5] = b.y;
-          w[6] = b.z;
-          w[7] = b.w;
-        }
-      } else if constexpr (BYTES == 8) {
-        const uint2* p = reinterpret_cast<const uint2*>(lo);
-        const uint2 a = __ldcs(p);
-        w[0] = a.x;
-        w[1] = a.y;
-        if constexpr (!AL) {
-          const uint2 b = two ? __ldcs(p + 1) : make_uint2(0u, 0u);
-          w[2] = b.x;
-          w[3] = b.y;
-        }
-      } else {
-        const unsigned* p = reinterpret_cast<const unsigned*>(lo);
-        w[0] = __ldcs(p);
-        if constexpr (!AL) w[1] = two ? __ldcs(p + 1) : 0u;
+    const uint64_t lo = AL ? ad : ad & ~(uint64_t)(BYTES - 1);
+    const bool two = !AL && (int)(ad - lo) + valid > BYTES;
+    if constexpr (BYTES == 16) {
+      const uint4* p = reinterpret_cast<const uint4*>(lo);
+      const uint4 a = __ldcs(p);
+      w[0] = a.x;
+      w[1] = a.y;
+      w[2] = a.z;
+      w[3] = a.w;
+      if constexpr (!AL) {
+        const uint4 b = two ? __ldcs(p + 1) : make_uint4(0u, 0u, 0u, 0u);
+        w[4] = b.x;
+        w[5] = b.y;
+        w[6] = b.z;
+        w[7] = b.w;
       }
+    } else if constexpr (BYTES == 8) {
+      const uint2* p = reinterpret_cast<const uint2*>(lo);
+      const uint2 a = __ldcs(p);
+      w[0] = a.x;
+      w[1] = a.y;
+      if constexpr (!AL) {
+        const uint2 b = two ? __ldcs(p + 1) : make_uint2(0u, 0u);
+        w[2] = b.x;
+        w[3] = b.y;
+      }
+    } else {
+      const unsigned* p = reinterpret_cast<const unsigned*>(lo);
+      w[0] = __ldcs(p);
+      if constexpr (!AL) w[1] = two ? __ldcs(p + 1) : 0u;
     }
   }
 
   // The window's words, for an address with the low bits k.
   template <bool AL, int ES>
   __device__ __forceinline__ void cut(uint32_t k) {
-    if constexpr (!AL && BYTES >= 4) {
+    if constexpr (!AL) {
       if constexpr (N == 4) {
         if (k & 8) {
 #pragma unroll
