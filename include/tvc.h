@@ -288,10 +288,15 @@ size_t tvc_quantise_workspace_size(int order, const int64_t* dims);
  * Device outputs (nullable): lambda_out (1 double), sweeps_out (1 int),
  * status_out (1 int: TVC_OK, TVC_ERR_ZERO_NORM or TVC_ERR_NONFINITE; on
  * either error the offending x_j keeps its previous value and the run
- * stops), lambda_hist (iters doubles: lambda of each completed sweep).
+ * stops; TVC_ERR_TIMEOUT when a barrier of the one-launch kernel gave up, see
+ * tvc_device_error), lambda_hist (iters doubles: lambda of each completed sweep).
  * A is streamed twice per sweep.  order >= 2.  Workspace: at least
  * hopm_workspace_size(order, dims, dtype) bytes of device memory, 256-byte
  * aligned; it holds the run's state, so concurrent runs need separate ones.
+ * Tensors up to about 100 MB run in one cooperative launch of 16 blocks to one
+ * per SM, by their size (a block fills its SM): on several streams, runs of more
+ * than about 0.25e6 elements in FP64 arithmetic or 1.2e6 in FP32 arithmetic follow
+ * one another, smaller ones overlap.
  */
 tvc_status hopm(const void* A, int order, const int64_t* dims, void* const* x, int iters, double tol,
                 double* lambda_out, int* sweeps_out, int* status_out, double* lambda_hist, tvc_dtype dtype,
@@ -347,7 +352,7 @@ size_t hopm_backward_workspace_size(int order, const int64_t* dims, tvc_dtype dt
  * y, gx and gA are formed from one read of A where the shape allows, else one
  * item kind per result), largest tensors first, and
  * pulled by persistent blocks from an atomic counter.  (hopm_batched runs
- * one thread-block cluster per tensor.)
+ * one thread-block cluster per tensor, one block per small tensor.)
  * All pointers in a descriptor are device pointers, FP32, dense row-major.
  */
 typedef struct {
@@ -385,7 +390,8 @@ size_t tvc_batched_workspace_size(const tvc_batch_desc* descs, int count);
 /* Times the candidate block mappings (lanes per output) of the forward
  * contraction of rows v == 1 on the tensors of each such shape class of the
  * batch and keeps the fastest for later calls of tvc_batched
- * in this process; synchronises the stream.
+ * in this process (tensors whose y shares a pass with gx do not use it);
+ * synchronises the stream.
  * workspace: tvc_batched_workspace_size(descs, count) bytes; a batch
  * uploaded on it before must be uploaded again (call without
  * TVC_BATCH_PREUPLOADED). */
@@ -393,7 +399,8 @@ tvc_status tvc_batched_autotune(const tvc_batch_desc* descs, int count, void* wo
                                 tvc_stream_t stream);
 
 /* `iters` Gauss-Seidel HOPM sweeps (Section 3, Algorithm 1's schedule) on
- * every tensor of the batch, one thread-block cluster per tensor; FP64 norms. */
+ * every tensor of the batch, one thread-block cluster (small tensors: one block)
+ * per tensor; FP64 norms. */
 tvc_status hopm_batched(const hopm_batch_desc* descs, int count, int iters, int flags, void* workspace,
                         size_t ws_bytes, tvc_stream_t stream);
 size_t hopm_batched_workspace_size(const hopm_batch_desc* descs, int count);

@@ -656,7 +656,8 @@ class TVCBatch:
 
 
 class HOPMBatch:
-    """A batch of FP32 power methods (one thread-block cluster per tensor, `iters` sweeps).
+    """A batch of FP32 power methods (a thread-block cluster or, for small tensors,
+    one block per tensor; `iters` sweeps).
     items: dicts with A (float32 CUDA tensor), x (its start vectors, updated
     in place) and any of lam, status; the batch holds on to them, since the
     uploaded descriptors keep their addresses."""

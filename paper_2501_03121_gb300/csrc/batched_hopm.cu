@@ -601,9 +601,9 @@ HLayout layout_hopm(const hopm_batch_desc* d, int count) {
   // block streams about 15 GB/s of it), narrower ones meet at fewer and
   // cheaper barriers.  Halve while the clusters resident at once would still
   // share the whole batch more evenly than its largest tensor: 10 sweeps of
-  // 512 tensors with 16 / 8 / 4 / 2 blocks 57 / 42 / 38 / 50 ms (rule: 4),
-  // 283 tensors 33 / 24 / 26 / 46 ms (8), 5 sweeps of 73 tensors 4.4 / 5.3 /
-  // 9.9 / 17 ms (16).
+  // 512 tensors with 16 / 8 / 4 / 2 blocks 51 / 36 / 33 / 49 ms (rule: 4),
+  // 283 tensors 32 / 22 / 26 / 46 ms (8), 5 sweeps of 73 tensors 4.1 / 5.2 /
+  // 9.5 / 18 ms (16).
   const int blocks = 2 * device_sms();
   int cl = 16;
   while (cl > 2 && 1.25 * (double)largest * (blocks / (cl / 2)) < (double)total) cl /= 2;
