@@ -240,7 +240,7 @@ __device__ __forceinline__ double gx_lanes(double (&a)[M]) {
 // / 47 / 84.  Single-double: 75 / 68 / 43 / 66.  A kernel that joined the lanes
 // in plain pairs after every piece took 80 / 84 / 44 / 73 on plain data, 336 /
 // 386 / 175 / 284 with 1% zeros or a small gy, and was up to nine times further
-// off (480x161 mode 0: 1.6e-14 of the terms' root sum of squares, 2.8e-15 here).
+// off (480x161 mode 0: 1.6e-14 of the terms' root sum of squares, 3.1e-15 here).
 template <tvc_dtype DT>
 inline constexpr int kGxTile = DT == TVC_F64 ? 4 : 2;  // pieces per thread and tile at most (48 KB of shared memory)
 constexpr int kGx64Rows = 128;                          // rows per chunk at most
